@@ -14,9 +14,10 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libweno.so")
-SOURCES = ["weno_kernels.cu", "weno_orders.cu", "weno_api.cu", "weno_noalloc.cu", "weno_engine.cu",
+SOURCES = ["weno_stage_tiny.cu", "weno_stage_fp32.cu", "weno_stage_noai.cu", "weno_stage_ai.cu",
+           "weno_kernels.cu", "weno_orders.cu", "weno_api.cu", "weno_noalloc.cu", "weno_engine.cu",
            "weno_peak.cu"]
-HEADERS = ["weno_device.cuh", "weno_tiles.cuh", "weno_tiles1d.cuh", "weno_internal.h"]
+HEADERS = ["weno_device.cuh", "weno_fixed.cuh", "weno_tiles.cuh", "weno_tiles1d.cuh", "weno_internal.h"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

@@ -17,6 +17,9 @@
 #pragma once
 #include <cstdint>
 
+#include "weno_fixed.cuh"
+#include "weno_internal.h"
+
 namespace weno {
 
 // Parameters of eqs. (21)-(22) for one characteristic field.  The field's
@@ -34,6 +37,8 @@ struct ReconParams {
   float mef;     // me^2 = eps / 9 = mef 2^eme, mef in [1, 2) (FP32)
   int eme;
   int lthr;      // dev >= 2^(lthr - 1019) implies me dev >= 2^30 mo (mo negligible)
+  int es_lo, es_hi;  // exponents of a field's largest difference the integer path takes
+  fx::Flt e3;        // 3 efix (no Ai), in the data's units squared
 };
 
 // ---------------------------------------------------------------------------
@@ -286,7 +291,7 @@ struct ZA6Part {
   double num, den;  // f = v2 + num / (6 den)
 };
 
-template <bool AI, bool P1>
+template <int AI, bool P1>
 __device__ __forceinline__ ZA6Part za6d(double d0, double d1, double d2, double d3, double d4,
                                         const ReconParams &P) {
   const double s0 = d1 - d0, s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3;
@@ -406,46 +411,93 @@ __device__ __forceinline__ double pair_flux(double base, const ZA6Part &p, const
   return fma(q, 1.0 / 6.0, base);
 }
 
-// One characteristic field of one face (FP64): w[j], g[j] are the projected
-// states and fluxes of the six stencil cells i-2 .. i+3 and A the field's GLF
-// speed.  The split of eq. (6) (kernel scaling: without the 1/2) is applied
-// to the differences: f+ = g + A w has differences dg + A dw, and the
-// mirrored f- = g - A w, read from i+3 down to i-2, has differences
-// A dw - dg in reverse order; the two centre values add up to
-// (g_i + g_{i+1}) - A (w_{i+1} - w_i).  Returns h = f^+ + f^- at i+1/2.
-template <bool AI, bool P1>
-__device__ __forceinline__ double field_flux(const double (&w)[6], const double (&g)[6], double A,
-                                             const ReconParams &P) {
-  double dp[5], dm[5], dw2 = 0.0;
-#pragma unroll
-  for (int j = 0; j < 5; ++j) {
-    const double dw = w[j + 1] - w[j], dg = g[j + 1] - g[j];
-    dp[j] = fma(A, dw, dg);
-    dm[4 - j] = fma(A, dw, -dg);
-    if (j == 2) dw2 = dw;
-  }
-  const double base = fma(-A, dw2, g[2] + g[3]);
-  return pair_flux(base, za6d<AI, P1>(dp[0], dp[1], dp[2], dp[3], dp[4], P),
-                   za6d<AI, P1>(dm[0], dm[1], dm[2], dm[3], dm[4], P));
-}
-
-// The same from the differences alone: dw[j] = w_{j+1} - w_j and
-// dg[j] = g_{j+1} - g_j over the six stencil cells.  Returns h less the
-// centre values g_i + g_{i+1}, i.e. the dissipation -A (w_{i+1} - w_i) plus
-// the two reconstructions' corrections; the caller adds the centre values
-// back (the 2D kernel in physical form after the back-projection, where
-// R (g_i + g_{i+1}) is the physical F_i + F_{i+1}).
-template <bool AI, bool P1>
-__device__ __forceinline__ double field_flux_d(const double (&dw)[5], const double (&dg)[5],
-                                               double A, const ReconParams &P) {
+// The two reconstructions of one field in FP64 from its differences: the path
+// of p != 1, and of magnitudes the integer path leaves out (a field whose
+// largest difference is below 2^-959, below mu_0, or not finite).
+template <int AI, bool P1>
+__device__ __noinline__ double pair_wide(double base, const double *dw, const double *dg, double A,
+                                         const ReconParams &P) {
   double dp[5], dm[5];
 #pragma unroll
   for (int j = 0; j < 5; ++j) {
     dp[j] = fma(A, dw[j], dg[j]);
     dm[4 - j] = fma(A, dw[j], -dg[j]);
   }
-  return pair_flux(-A * dw[2], za6d<AI, P1>(dp[0], dp[1], dp[2], dp[3], dp[4], P),
-                   za6d<AI, P1>(dm[0], dm[1], dm[2], dm[3], dm[4], P));
+  return pair_flux(base, za6d<(AI != kNoAi), P1>(dp[0], dp[1], dp[2], dp[3], dp[4], P),
+                   za6d<(AI != kNoAi), P1>(dm[0], dm[1], dm[2], dm[3], dm[4], P));
+}
+
+// The sensitivity term of recon6 for one stencil (see there), in its units:
+// constant without the descaler, else 3 (sqrt(4 eps) mu)^2 from the mean
+// deviation of the stencil in FP64.
+template <int AI>
+__device__ __forceinline__ fx::Flt sens_fixed(const fx::i64 (&d)[5], int es,
+                                              const ReconParams &P) {
+  fx::Flt e = P.e3;
+  if constexpr (AI == kAi) {
+    const double d0 = (double)d[0], d1 = (double)d[1], d2 = (double)d[2], d3 = (double)d[3],
+                 d4 = (double)d[4];
+    const double a0 = -(d0 + d1), a1 = -d1, a3 = d2, a4 = d2 + d3, a5 = a4 + d4;
+    const double m = ((a0 + a1) + (a3 + a4) + a5) * (1.0 / 6.0);
+    const double dev = fabs(a0 - m) + fabs(a1 - m) + fabs(m) + fabs(a3 - m) + fabs(a4 - m) +
+                       fabs(a5 - m);
+    const double unit = __longlong_as_double((long long)(es - 56) << 52);  // 2^(es - 1079)
+    const double sm = fma(dev * unit, P.me, P.mo);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(3.0 * (sm * sm));
+    e.m = (b << 11) | 0x8000000000000000ull;
+    e.e = (int)(b >> 52) - 1086;
+  }
+  e.e -= 2 * (es - 1079);
+  return e;
+}
+
+// One characteristic field of one face (FP64) from the differences dw[j] =
+// w_{j+1} - w_j, dg[j] = g_{j+1} - g_j of its projected states and fluxes over
+// the six stencil cells; A is the field's GLF speed.  The split of eq. (6)
+// (kernel scaling: without the 1/2) is applied to the differences: f+ = g + A w
+// has differences dg + A dw, and the mirrored f- = g - A w, read from i+3 down
+// to i-2, has differences A dw - dg in reverse order.  Returns
+// h = f^+ + f^- at i+1/2 with centre = g_i + g_{i+1}, or h less those centre
+// values with centre = 0 (the Euler kernels add them back in physical form
+// after the back-projection, where R (g_i + g_{i+1}) is F_i + F_{i+1}).
+// For p = 1 the two reconstructions run on the integer pipes (recon6 in
+// weno_fixed.cuh) in units of the ten differences' largest exponent; what is
+// left to FP64 is A dw, the sum's conversion and its scaling: 7 operations a
+// field instead of 120.  A field that does not vary at all needs neither.
+template <int AI, bool P1>
+__device__ __forceinline__ double field_flux(const double (&dw)[5], const double (&dg)[5],
+                                             double A, const ReconParams &P, double centre) {
+  double xw[5];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) xw[j] = __dmul_rn(A, dw[j]);
+  const double base = __dsub_rn(centre, xw[2]);
+  if constexpr (P1) {
+    const int es = fx::top_exponent(xw, dg);
+    if (es >= P.es_lo && es <= P.es_hi) {
+      fx::i64 p[5], n[5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const fx::i64 x = fx::to_fixed(xw[j], es), g = fx::to_fixed(dg[j], es);
+        p[j] = x + g;
+        n[4 - j] = x - g;
+      }
+      fx::i64 c;
+      if constexpr (AI == kAiTiny) {
+        c = fx::recon6<false>(p[0], p[1], p[2], p[3], p[4], P.e3) +
+            fx::recon6<false>(n[0], n[1], n[2], n[3], n[4], P.e3);
+      } else {
+        c = fx::recon6<true>(p[0], p[1], p[2], p[3], p[4], sens_fixed<AI>(p, es, P)) +
+            fx::recon6<true>(n[0], n[1], n[2], n[3], n[4], sens_fixed<AI>(n, es, P));
+      }
+      return __fma_rn((double)c, fx::scale_back(es), base);
+    }
+    unsigned long long any = 0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j)
+      any |= (unsigned long long)(__double_as_longlong(xw[j]) | __double_as_longlong(dg[j])) << 1;
+    if (any == 0) return base;
+  }
+  return pair_wide<AI, P1>(base, dw, dg, A, P);
 }
 
 // ---------------------------------------------------------------------------
@@ -576,7 +628,7 @@ struct RPart {
   double vc, num, den;
 };
 
-template <int R, bool AI, bool P1>
+template <int R, int AI, bool P1>
 __device__ __forceinline__ RPart za_r(const double (&v)[2 * R], const ReconParams &P) {
   using Tb = OrderTab<R>;
   constexpr int N = 2 * R;
@@ -843,7 +895,7 @@ __device__ __forceinline__ double field_flux_f32(const double (&w)[6], const dou
 }
 
 // field_flux_f32 from the differences alone, less the centre values
-// g_i + g_{i+1} (as field_flux_d).
+// g_i + g_{i+1} (as field_flux with centre = 0).
 template <bool P1>
 __device__ __forceinline__ double field_flux_f32d(const double (&dw)[5], const double (&dg)[5],
                                                   double A, const Recon32 &P) {

@@ -1,0 +1,249 @@
+// weno_fixed.cuh -- the sixth-order reconstruction of eqs. (11)-(22) on the
+// integer pipes.
+//
+// What bounds the stage kernels is FP64 issue: an SM of GB300 starts about
+// 1.95 FP64 operations per clock, but (measured) 62 integer multiply-adds
+// (58 with a 64-bit result) and beside them 62 logic or shift operations, or
+// 118 additions.  A 64-bit integer step therefore costs a few percent of an
+// FP64 one, and the reconstruction -- 71 % of the FP64 work of a 2D stage when
+// it ran there -- needs neither FP64's range inside a stencil nor its
+// rounding: it is homogeneous of degree one, its answer is an average of
+// candidates within the stencil's variation, and so an error of a few units
+// of 2^-57 of the largest difference, in every difference, is below the
+// rounding FP64 gives it (2^-53 per operation).
+//
+// Number formats (tests/test_kernel_fixed.py restates them and measures the
+// error against quadruple precision):
+//  * differences and what is linear in them (second differences, candidate
+//    fluxes, the fifth difference): 64-bit integers in units of 2^-57 of the
+//    power of two above the largest of the ten differences of a field -- exact
+//    sums;
+//  * indicators and tau: a 64-bit mantissa with its top bit set and an
+//    exponent;
+//  * weights: their reciprocals 1/b_k and 1/(4 tau), aligned to the largest,
+//    since alpha_k of eqs. (20)-(21) is proportional to d_k (1/b_k + 1/(4 tau))
+//    for p = 1: a weighted mean needs its weights to a fixed fraction of the
+//    largest one only.
+#pragma once
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#define WENO_FX __device__ __forceinline__
+#else
+#include <cmath>
+#define WENO_FX inline
+#endif
+
+namespace weno {
+namespace fx {
+
+typedef unsigned long long u64;
+typedef long long i64;
+
+#ifdef __CUDA_ARCH__
+// 64-bit shifts that give 0 for a count of 64 or more
+WENO_FX u64 shr(u64 x, int n) {
+  u64 r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+WENO_FX u64 shl(u64 x, int n) {
+  u64 r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));
+  return r;
+}
+WENO_FX int clz32(uint32_t x) { return __clz((int)x); }
+WENO_FX uint32_t rcp_seed(uint32_t fbits) {  // bits of about 1 / f, f in [1, 2)
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(fbits)));
+  return __float_as_uint(r);
+}
+WENO_FX u64 dbits(double x) { return (u64)__double_as_longlong(x); }
+WENO_FX double bitsd(u64 b) { return __longlong_as_double((i64)b); }
+#else
+WENO_FX u64 shr(u64 x, int n) { return n >= 64 ? 0 : x >> n; }
+WENO_FX u64 shl(u64 x, int n) { return n >= 64 ? 0 : x << n; }
+WENO_FX int clz32(uint32_t x) { return x ? __builtin_clz(x) : 32; }
+WENO_FX uint32_t rcp_seed(uint32_t fbits) {
+  float f, r;
+  std::memcpy(&f, &fbits, 4);
+  r = 1.0f / f;
+  std::memcpy(&fbits, &r, 4);
+  return fbits;
+}
+WENO_FX u64 dbits(double x) {
+  u64 b;
+  std::memcpy(&b, &x, 8);
+  return b;
+}
+WENO_FX double bitsd(u64 b) {
+  double x;
+  std::memcpy(&x, &b, 8);
+  return x;
+}
+#endif
+
+WENO_FX uint32_t lo32(u64 x) { return (uint32_t)x; }
+WENO_FX uint32_t hi32(u64 x) { return (uint32_t)(x >> 32); }
+WENO_FX u64 abs64(i64 x) { return x < 0 ? 0 - (u64)x : (u64)x; }
+
+// a b / 2^64, low by at most 2 (the product of the low words and the carries
+// out of the lower 64 bits are left out): three multiply-adds.
+WENO_FX u64 mulhi64(u64 a, u64 b) {
+  const u64 c1 = (u64)hi32(a) * lo32(b), c2 = (u64)lo32(a) * hi32(b);
+  return (u64)hi32(a) * hi32(b) + hi32(c1) + hi32(c2);
+}
+// a^2 / 2^64 for a < 2^63.
+WENO_FX u64 sqrhi(u64 a) {
+  const u64 c = (u64)(hi32(a) * 2u) * lo32(a);
+  return (u64)hi32(a) * hi32(a) + hi32(c);
+}
+
+// Leading zeros of a 64-bit number (64 for 0) with one FLO.
+WENO_FX int clz64(u64 x) {
+  const uint32_t h = hi32(x), w = h ? h : lo32(x);
+  return clz32(w) + (h ? 0 : 32);
+}
+
+// 2^127 / X for X >= 2^63, low by at most 2^-60 of it and never high (so it
+// stays below 2^64): the
+// special-function unit's FP32 reciprocal of the top 24 bits, taken a little
+// low so that e = 1 - x r is positive (0 < e < 2^-20), then r (1 + e + e^2)
+// in 64-bit arithmetic.
+WENO_FX u64 rcp64(u64 X) {
+  const uint32_t rb = rcp_seed((hi32(X) >> 8) | 0x3F000001u);
+  const uint32_t r = rb * 256u + (0x80000000u - 0x400u);  // r / 2^32 < 1 / x, x = X / 2^63
+  const u64 d = (u64)hi32(X) * r + hi32((u64)lo32(X) * r);  // x r in units of 2^-63
+  const u64 e = 0x7FFFFFFFFFFFFFFFull - d;          // a unit low, for what d leaves out
+  const uint32_t eh = (uint32_t)(e >> 12);          // e in units of 2^-51 (31 bits)
+  const u64 g = e + (hi32((u64)eh * eh) >> 7);      // + e^2: 2^-102+32 = 2^-70 -> 2^-63
+  const u64 w = (u64)r * lo32(g);
+  return ((u64)r * (0x80000000u + hi32(g)) + hi32(w)) << 1;
+}
+
+// Fixed-point value of x: x 2^(57 - (es - 1022)), truncated towards zero, with
+// es at least the biased exponent of x and at least 64 (then a zero x, and
+// any x below 2^-57 of the unit, gives 0).
+WENO_FX i64 to_fixed(double x, int es) {
+  const u64 b = dbits(x);
+  const u64 m = (b << 11) | 0x8000000000000000ull;
+  const int e = (int)((b >> 52) & 0x7FF);
+  const u64 v = shr(m, 7 + es - e);
+  return (i64)b < 0 ? -(i64)v : (i64)v;
+}
+
+// 13 s^2 + 3 t^2 = 3 (4 beta) of |s|, |t| < 2^62, as raw 2^(64 - 2 n).
+struct Ind {
+  u64 raw;  // 0 or at least 2^59.5
+  int n;
+};
+WENO_FX Ind indicator(i64 s, i64 t) {
+  const u64 sa = abs64(s), ta = abs64(t);
+  Ind o;
+  o.n = clz64(sa | ta) - 2;
+  const u64 S = sqrhi(shl(sa, o.n)), T = sqrhi(shl(ta, o.n));
+  o.raw = 13ull * S + 3ull * T;
+  return o;
+}
+
+// A positive number m 2^e with the top bit of m set.
+struct Flt {
+  u64 m;
+  int e;
+};
+// raw 2^e, raw = 0 or above 2^57; a zero becomes 2^(63 + e0).
+WENO_FX Flt normal(u64 raw, int e, int e0) {
+  Flt f;
+  const int n = clz32(hi32(raw));
+  const bool z = raw == 0;
+  f.m = z ? 0x8000000000000000ull : shl(raw, n);
+  f.e = z ? e0 : e - n;
+  return f;
+}
+// raw 2^e + s, aligned to the larger of the two.
+WENO_FX Flt normal_plus(u64 raw, int e, const Flt &s) {
+  const int d = raw ? s.e - e : 8192;
+  const u64 v = shr(raw, d > 0 ? d + 1 : 1) + shr(s.m, d > 0 ? 1 : 1 - d);
+  return normal(v, (d > 0 ? s.e : e) + 1, 0);
+}
+
+// Six times the correction f - v2 of eqs. (14)-(22) (p = 1) of the stencil
+// with differences d_j, |d_j| < 2^58, in their units:
+//   c = r_1 + sum_k w_k (r_k - r_1), w_k = D_k z_k / sum D_j z_j,
+//   z_k = 1/b_k + 1/T, b_k = 3 (4 beta_k), T = 3 (4 tau), D = (1, 9, 9, 1).
+// SENS: whether the sensitivity term e = 3 (4 eps mu^2) of eq. (21) is added
+// to the b_k.  At epsilon <= 2^-126 it is below a quarter of the unit squared
+// wherever mu_0 is below the largest difference, and it could only decide
+// between candidates that agree to a few units; it is then left out, and an
+// indicator that is 0 in these units counts as 2^-10.
+template <bool SENS>
+WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e) {
+  const i64 s0 = d1 - d0, s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3;
+  const Ind i0 = indicator(s0, 2 * d1 + s0);           // t_0 = 3 d1 - d0
+  const Ind i1 = indicator(s1, d1 + d2);               // t_1
+  const Ind i2 = indicator(s2, 2 * d2 - s2);           // t_2 = 3 d2 - d3
+  const Ind id = indicator(s3, s3 + 2 * (s3 - d3));    // t_3 = 3 d4 - 5 d3
+  const i64 q = s1 - s2;
+  const i64 r5 = (s3 - s0) + 3 * q;                    // fifth difference
+  // b_3 = mean of the four (eq. (16)), aligned to the largest
+  const int a01 = i0.n < i1.n ? i0.n : i1.n, a2d = i2.n < id.n ? i2.n : id.n;
+  const int nm = a01 < a2d ? a01 : a2d;
+  const u64 raw3 = shr(i0.raw, 2 * (i0.n - nm) + 2) + shr(i1.raw, 2 * (i1.n - nm) + 2) +
+                   shr(i2.raw, 2 * (i2.n - nm) + 2) + shr(id.raw, 2 * (id.n - nm) + 2);
+  Flt b0, b1, b2, b3;
+  if (SENS) {
+    b0 = normal_plus(i0.raw, 64 - 2 * i0.n, e);
+    b1 = normal_plus(i1.raw, 64 - 2 * i1.n, e);
+    b2 = normal_plus(i2.raw, 64 - 2 * i2.n, e);
+    b3 = normal_plus(raw3, 64 - 2 * nm, e);
+  } else {
+    b0 = normal(i0.raw, 64 - 2 * i0.n, -73);
+    b1 = normal(i1.raw, 64 - 2 * i1.n, -73);
+    b2 = normal(i2.raw, 64 - 2 * i2.n, -73);
+    b3 = normal(raw3, 64 - 2 * nm, -73);
+  }
+  // T = 12 r5^2
+  const u64 ra = abs64(r5);
+  const int nt = clz64(ra) - 1;
+  const u64 sq = sqrhi(shl(ra, nt));
+  const Flt T = normal(3ull * sq, 66 - 2 * nt, -16384);  // 0: far below every b_k
+  // y_k = D_k z_k with the largest of D_k / b_k and 8 / T in [2^60, 2^61)
+  const int e0 = b0.e < b3.e ? b0.e : b3.e, e1 = (b1.e < b2.e ? b1.e : b2.e) - 3;
+  const int e01 = e0 < e1 ? e0 : e1, em = (e01 < T.e - 3 ? e01 : T.e - 3) - 3;
+  const u64 w8 = shr(rcp64(T.m), T.e - 3 - em), w1 = w8 >> 3, w9 = w8 + w1;  // 8/T, 1/T, 9/T
+  const u64 v1 = shr(rcp64(b1.m), b1.e - 3 - em), v2 = shr(rcp64(b2.m), b2.e - 3 - em);
+  const u64 z0 = shr(rcp64(b0.m), b0.e - em) + w1, z3 = shr(rcp64(b3.m), b3.e - em) + w1;
+  const u64 z1 = v1 + (v1 >> 3) + w9, z2 = v2 + (v2 >> 3) + w9;
+  const u64 den = (z0 + z3) + (z1 + z2);  // < 6.75 2^61
+  // sum_k D_k z_k (r_k - r_1) / den with the sum formed on r_k - r_1 + 2^62 >= 0
+  const int nd = clz32(hi32(den));
+  const u64 y0 = shl(z0, nd), y2 = shl(z2, nd), y3 = shl(z3, nd);  // y0 + y2 + y3 < 2^64
+  const i64 p0 = 2 * (s0 - s1), p3 = q + 2 * (s3 - s2);
+  const u64 B = 0x8000000000000000ull;
+  const u64 N = mulhi64(y0, B + 2 * (u64)p0) + mulhi64(y2, B + 2 * (u64)q) +
+                mulhi64(y3, B + 2 * (u64)p3);
+  const i64 Ns = (i64)(N - (y0 >> 1) - (y2 >> 1) - (y3 >> 1));
+  const u64 c = mulhi64(abs64(Ns), rcp64(shl(den, nd)));
+  return (d1 + 2 * d2) + (Ns < 0 ? -(i64)c : (i64)c);
+}
+
+// The largest biased exponent of the ten differences.
+WENO_FX int top_exponent(const double (&xw)[5], const double (&dg)[5]) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const uint32_t a = hi32(dbits(xw[j])) & 0x7FFFFFFFu, b = hi32(dbits(dg[j])) & 0x7FFFFFFFu;
+    m = m > a ? m : a;
+    m = m > b ? m : b;
+  }
+  return (int)(m >> 20);
+}
+
+// c 2^(es - 1022 - 57) / 6: a correction of recon6 back in the data's units.
+WENO_FX double scale_back(int es) {
+  return bitsd(dbits(1.0 / 6.0) + ((u64)(i64)(es - 1079) << 52));
+}
+
+}  // namespace fx
+}  // namespace weno

@@ -5,6 +5,12 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#ifdef __CUDACC__
+#define WENO_HD __host__ __device__
+#else
+#define WENO_HD
+#endif
+
 namespace weno {
 
 // Device status word and the location of the first failure.
@@ -16,6 +22,24 @@ struct DevStatus {
 
 // 2D tile variants of the single-problem stage kernel (see launch_stage_t).
 constexpr int kTileVariants = 11;
+
+// Weight modes (template parameter AI): without the descaler of eq. (22),
+// with it, and with it where the sensitivity term eps mu^2 lies below the
+// resolution of the integer path (eps <= 2^-126 and mu_0 <= 2^-100, the
+// paper's 1e-40 among them), which then skips mu altogether.
+enum { kNoAi = 0, kAi = 1, kAiTiny = 2 };
+WENO_HD inline int weight_mode(bool ai, double eps, double mu0) {
+  return !ai ? kNoAi : (eps <= 0x1p-126 && mu0 <= 0x1p-100 ? kAiTiny : kAi);
+}
+
+// Tile shapes are built in full for the default weights and for the FP32
+// reconstruction with p = 1; the other modes map every shape to one of three.
+WENO_HD constexpr bool all_tile_shapes(int mode, bool p1, int precision) {
+  return p1 && (mode == kAiTiny || precision == 1);
+}
+WENO_HD constexpr int tile_shape_built(bool all, int v) {
+  return all ? v : (v == 8 ? 8 : (v == 2 || v == 4 || v == 7 ? 2 : 9));
+}
 
 // Everything one stage launch needs (passed by value).
 struct StageArgs {
@@ -121,6 +145,12 @@ bool encode_state_map(const double *U, long long nbatch, long long ny, long long
 
 cudaError_t launch_alpha(const AlphaArgs &a, cudaStream_t s);
 cudaError_t launch_stage(const StageArgs &a, cudaStream_t s);
+// The sixth-order launches by weight mode, each in its own translation unit so
+// they compile in parallel: the default weights, FP32 reconstruction, the rest.
+cudaError_t launch_stage_tiny(const StageArgs &a, cudaStream_t s);
+cudaError_t launch_stage_fp32(const StageArgs &a, cudaStream_t s);
+cudaError_t launch_stage_noai(const StageArgs &a, cudaStream_t s);
+cudaError_t launch_stage_ai(const StageArgs &a, cudaStream_t s);
 // The same for a.order_r = 2, 4, 5 (FP64 reconstruction only).
 cudaError_t launch_stage_orders(const StageArgs &a, cudaStream_t s);
 // alpha bits -> doubles, and the CFL dt per problem

@@ -1,8 +1,7 @@
-// weno_kernels.cu -- sixth-order (WENO-ZA6) stage launches, the wavespeed
-// reductions of eq. (6), the serving engine's persistent stage kernel and the
-// host-side launchers for GB300 (sm_103a).  The tile kernels themselves are in
-// weno_tiles.cuh; the schemes of other orders are instantiated in
-// weno_orders.cu.
+// weno_kernels.cu -- the wavespeed reductions of eq. (6), the serving engine's
+// persistent stage kernel and the host-side launchers for GB300 (sm_103a).
+// The tile kernels themselves are in weno_tiles.cuh, instantiated by weight
+// mode in weno_stage_*.cu (sixth order) and by order in weno_orders.cu.
 #include <mutex>
 
 #include "weno_tiles.cuh"
@@ -178,26 +177,25 @@ __global__ void __launch_bounds__(kEngineThreads, kEngineBlocksPerSM) k_engine(c
     const SlotDev &S = e.slots[t.slot];
     if (S.active) {
       const StageArgs a = slot_stage_args(S, e.stage);
+      const bool tiny = weight_mode(true, S.eps, S.mu0) == kAiTiny;
       if (S.ndim == 2) {
         if (S.precision == 1)
-          euler2d_tile<kEngineTX, kEngineTY, true, true, 1>(a, 0, t.tile, t.tile == 0, sm);
+          euler2d_tile<kEngineTX, kEngineTY, kAi, true, 1>(a, 0, t.tile, t.tile == 0, sm);
+        else if (tiny)
+          euler2d_tile<kEngineTX, kEngineTY, kAiTiny, true, 0>(a, 0, t.tile, t.tile == 0, sm);
         else
-          euler2d_tile<kEngineTX, kEngineTY, true, true, 0>(a, 0, t.tile, t.tile == 0, sm);
+          euler2d_tile<kEngineTX, kEngineTY, kAi, true, 0>(a, 0, t.tile, t.tile == 0, sm);
       } else {
         if (S.precision == 1)
-          line1d_tile<3, true, true, 1, kEngine1DCells>(a, 0, t.tile, t.tile == 0, sm);
+          line1d_tile<3, kAi, true, 1, kEngine1DCells>(a, 0, t.tile, t.tile == 0, sm);
+        else if (tiny)
+          line1d_tile<3, kAiTiny, true, 0, kEngine1DCells>(a, 0, t.tile, t.tile == 0, sm);
         else
-          line1d_tile<3, true, true, 0, kEngine1DCells>(a, 0, t.tile, t.tile == 0, sm);
+          line1d_tile<3, kAi, true, 0, kEngine1DCells>(a, 0, t.tile, t.tile == 0, sm);
       }
     }
     __syncthreads();
   }
-}
-
-template <bool AI, bool P1>
-cudaError_t launch_order(const StageArgs &a, cudaStream_t s) {
-  if (a.order_r != 3) return launch_stage_orders(a, s);  // weno_orders.cu
-  return launch_stage_t<AI, P1, 0, 3>(a, s);
 }
 
 }  // namespace
@@ -241,11 +239,11 @@ bool encode_state_map(const double *U, long long nbatch, long long ny, long long
 }
 
 cudaError_t launch_stage(const StageArgs &a, cudaStream_t s) {
-  const bool p1 = (a.p == 1.0);
-  if (a.precision == 1)  // FP32 reconstruction (affine-invariant weights, order 6)
-    return p1 ? launch_stage_t<true, true, 1, 3>(a, s) : launch_stage_t<true, false, 1, 3>(a, s);
-  if (a.ai) return p1 ? launch_order<true, true>(a, s) : launch_order<true, false>(a, s);
-  return p1 ? launch_order<false, true>(a, s) : launch_order<false, false>(a, s);
+  if (a.order_r != 3) return launch_stage_orders(a, s);  // weno_orders.cu
+  if (a.precision == 1) return launch_stage_fp32(a, s);
+  const int mode = weight_mode(a.ai != 0, a.eps, a.mu0);
+  if (mode == kAiTiny && a.p == 1.0) return launch_stage_tiny(a, s);
+  return mode == kNoAi ? launch_stage_noai(a, s) : launch_stage_ai(a, s);
 }
 
 size_t engine_smem_bytes() {

@@ -7,7 +7,7 @@
 namespace weno {
 namespace {
 
-template <bool AI, bool P1>
+template <int AI, bool P1>
 cudaError_t launch_r(const StageArgs &a, cudaStream_t s) {
   switch (a.order_r) {
     case 2: return launch_stage_t<AI, P1, 0, 2>(a, s);

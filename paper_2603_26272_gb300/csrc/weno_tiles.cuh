@@ -159,6 +159,18 @@ __device__ __forceinline__ ReconParams make_rp(const StageArgs &a, double k) {
   } else {
     r.lthr = -(1 << 20);
   }
+  // the integer path: exponents from 64 up (to_fixed) and, where it leaves the
+  // sensitivity term out, from a largest difference of scale mu_0 up; squares
+  // of differences up to 2^400 in the sensitivity term's FP64
+  const bool tiny = a.ai && a.eps <= 0x1p-126 && a.mu0 <= 0x1p-100;
+  r.es_hi = tiny ? 2046 : 1023 + 400;
+  r.es_lo = 64;
+  if (tiny) r.es_lo = max(64, ((__double2hiint(k * a.mu0) >> 20) & 0x7FF) + 1);
+  const double e3 = fmax(3.0 * r.efix, DBL_MIN);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(e3);
+  r.e3.m = (b << 11) | 0x8000000000000000ull;
+  r.e3.e = (int)(b >> 52) - 1086;
+  if (!tiny && (b >> 52) >= 2047) r.es_lo = 4096;
   return r;
 }
 
@@ -422,7 +434,7 @@ __host__ __device__ constexpr size_t smem_euler2d_tma() {
 // sm: dynamic shared memory of smem_euler2d_tma<TX, TY, R>() bytes.
 // tm: tensor map of the stage input as [nbatch * 4][ny][nx] doubles, or NULL
 // (plain loads only; the serving engine and tiles of launches without one).
-template <int TX, int TY, bool AI, bool P1, int PREC, int R>
+template <int TX, int TY, int AI, bool P1, int PREC, int R>
 __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b, long long tile,
                                                  bool zeroing_block, double *sm,
                                                  const CUtensorMap *tm) {
@@ -566,7 +578,7 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
 //
 // The reconstruction of a face needs, per characteristic field, only the
 // differences of the split fluxes f+- = g +- alpha w over its six stencil
-// cells (field_flux_d), and those are L (F_{j+1} - F_j) +- alpha L (U_{j+1}
+// cells (field_flux), and those are L (F_{j+1} - F_j) +- alpha L (U_{j+1}
 // - U_j): the face's left eigenvectors applied to differences of the state
 // and of the physical flux between adjacent cells.  Those differences are
 // formed once per cell pair and direction and shared by the five faces whose
@@ -592,7 +604,7 @@ __device__ __forceinline__ void normal_flux(double rho, double mn, double mt, do
   F3 = H * mn;
 }
 
-template <int TX, int TY, bool AI, bool P1, int PREC, int DIR>
+template <int TX, int TY, int AI, bool P1, int PREC, int DIR>
 __device__ __forceinline__ void tile6_sweep(const StageArgs &a, long long b, long long i0,
                                             long long j0, double gm1, double *sm,
                                             const ReconParams &rp2, const ReconParams &rp4) {
@@ -700,10 +712,10 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, long long b, lon
       h3 = field_flux_f32d<P1>(dw[2], dg[2], A3, r32);
       h4 = field_flux_f32d<P1>(dw[3], dg[3], A4, r32);
     } else {
-      h1 = field_flux_d<AI, P1>(dw[0], dg[0], A1, rp4);
-      h2 = field_flux_d<AI, P1>(dw[1], dg[1], A2, rp2);
-      h3 = field_flux_d<AI, P1>(dw[2], dg[2], A3, rp2);
-      h4 = field_flux_d<AI, P1>(dw[3], dg[3], A4, rp4);
+      h1 = field_flux<AI, P1>(dw[0], dg[0], A1, rp4, 0.0);
+      h2 = field_flux<AI, P1>(dw[1], dg[1], A2, rp2, 0.0);
+      h3 = field_flux<AI, P1>(dw[2], dg[2], A3, rp2, 0.0);
+      h4 = field_flux<AI, P1>(dw[3], dg[3], A4, rp4, 0.0);
     }
     double F0, F1, F2, F3;
     backproject4(fs, h1, h2, h3, h4, F0, F1, F2, F3);
@@ -730,7 +742,7 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, long long b, lon
 
 // One tile of a sixth-order 2D stage (see above).  sm: smem_euler2d<TX, TY>()
 // bytes; tm: tensor map of the stage input or NULL, as for euler2d_tile_gen.
-template <int TX, int TY, bool AI, bool P1, int PREC>
+template <int TX, int TY, int AI, bool P1, int PREC>
 __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, long long tile,
                                               bool zeroing_block, double *sm_in,
                                               const CUtensorMap *tm) {
@@ -817,7 +829,7 @@ __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, l
 
 // One tile of a 2D stage of order 2R (sixth order: euler2d_tile6; 4, 8, 10:
 // euler2d_tile_gen).
-template <int TX, int TY, bool AI, bool P1, int PREC, int R = 3>
+template <int TX, int TY, int AI, bool P1, int PREC, int R = 3>
 __device__ __forceinline__ void euler2d_tile(const StageArgs &a, long long b, long long tile,
                                              bool zeroing_block, double *sm,
                                              const CUtensorMap *tm = nullptr) {
@@ -829,7 +841,7 @@ __device__ __forceinline__ void euler2d_tile(const StageArgs &a, long long b, lo
 
 // MINB: resident blocks per SM the register allocation must allow.
 // tm: tensor map of a.Uin (see euler2d_tile), used when a.use_tma is set.
-template <int TX, int TY, int NT, int MINB, bool AI, bool P1, int PREC, int R = 3>
+template <int TX, int TY, int NT, int MINB, int AI, bool P1, int PREC, int R = 3>
 __global__ void __launch_bounds__(NT, MINB)
     k_euler2d(const StageArgs a, const __grid_constant__ CUtensorMap tm) {
   extern __shared__ __align__(128) double sm[];
@@ -857,7 +869,7 @@ inline int sm_count() {
 // less 1 KB the hardware keeps per block).
 constexpr size_t kSmemPerSM = 233472;
 
-template <int TX, int TY, int NT, int MINB, bool AI, bool P1, int PREC, int R = 3>
+template <int TX, int TY, int NT, int MINB, int AI, bool P1, int PREC, int R = 3>
 cudaError_t launch_2d(const StageArgs &a_in, cudaStream_t s) {
   StageArgs a = a_in;
   // TMA staging when the box fits beside the tile's planes at this
@@ -879,7 +891,7 @@ cudaError_t launch_2d(const StageArgs &a_in, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <bool AI, bool P1, int PREC, int R>
+template <int AI, bool P1, int PREC, int R>
 cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
   if (a.ndim == 2) {
     // tile variants (cells / threads / blocks per SM the registers allow):
@@ -896,10 +908,19 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     // same SM sub-partition, so an uneven count leaves three of the four
     // FP64 pipes idle at the end of a sweep): 9 = 16x15 / 128 / 3 (255 and
     // 256 faces), 10 = 14x17 / 128 / 3 (255 and 252).
+    // Weights other than the default ones (without Ai, with a sensitivity term
+    // that counts, p != 1) are built in three of the shapes (2, 8, 9; see
+    // tile_shape_built), which keeps the library's build short.
     // The other orders use 16x16 / 128 only, 3 blocks per SM at r = 2 and 2
     // at r = 4, 5 (their wider stencils need more registers).
     if constexpr (R != 3) {  // r = 2 fits the 168-register cap of 3 blocks per SM
       return launch_2d<16, 16, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
+    } else if constexpr (!all_tile_shapes(AI, P1, PREC)) {
+      switch (tile_shape_built(false, a.tile_variant)) {
+        case 2: return launch_2d<16, 8, 64, 4, AI, P1, PREC>(a, s);
+        case 8: return launch_2d<8, 8, 128, 2, AI, P1, PREC>(a, s);
+        default: return launch_2d<16, 15, 128, 3, AI, P1, PREC>(a, s);
+      }
     } else {
       switch (a.tile_variant) {
         case 1: return launch_2d<16, 16, 128, 2, AI, P1, PREC>(a, s);

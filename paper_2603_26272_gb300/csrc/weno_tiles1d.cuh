@@ -38,7 +38,7 @@ constexpr size_t smem_line1d() {
 // positive and the negative flux; blockDim >= 2 (T + 1)).  Every lane layout
 // runs the same arithmetic per field, so the results are bitwise identical.
 // sm: dynamic shared memory of smem_line1d<NC, T, R, LANES>() bytes.
-template <int NC, bool AI, bool P1, int PREC, int T, int R = 3, int LANES = 1>
+template <int NC, int AI, bool P1, int PREC, int T, int R = 3, int LANES = 1>
 __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, long long tile,
                                             bool zeroing_block, double *sm) {
   static_assert(R == 3 || PREC == 0, "FP32 reconstruction is sixth order only");
@@ -135,7 +135,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
       if constexpr (PREC == 1)
         h = field_flux_f32d<P1>(dW, dG, A, s_r32);
       else
-        h = field_flux_d<AI, P1>(dW, dG, A, s_rp[q == 1 ? 0 : 1]);
+        h = field_flux<AI, P1>(dW, dG, A, s_rp[q == 1 ? 0 : 1], 0.0);
       hb[3 * f + q] = h;
     }
     __syncthreads();
@@ -149,31 +149,49 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     }
   } else if constexpr (LANES == 2) {
     // the positive (even lane) and the mirrored negative flux (odd lane) of a
-    // scalar face; the partial sums meet by a lane shuffle
-    // (the differences and the centre sum as field_flux forms them)
+    // scalar face, the operations of field_flux: the corrections meet by a lane
+    // shuffle; a face off the integer path is left to the even lane alone
     const int f = tid >> 1, sgn = tid & 1;
     const bool act = (f <= T) && (i0 + f - 1 < nx);
-    ZA6Part part = {0.0, 1.0};
-    double base = 0.0;
+    double dw[5] = {}, dg[5] = {}, xw[5] = {};
+    double A = 0.0, centre = 0.0;
+    int es = 0;
+    fx::i64 c = 0;
+    const ReconParams &rp = s_rp[0];
     if (act) {
-      const double A = scalar_alpha_of(a.system, a.adv_speed, a.ustar, a.alpha_in + b * 8);
-      const ReconParams rp = s_rp[0];
-      double dd[5], dw2 = 0.0;
+      A = scalar_alpha_of(a.system, a.adv_speed, a.ustar, a.alpha_in + b * 8);
 #pragma unroll
       for (int j = 0; j < 5; ++j) {
-        const double dw = pl[0][f + j + 1] - pl[0][f + j], dg = pl[1][f + j + 1] - pl[1][f + j];
-        if (sgn)
-          dd[4 - j] = fma(A, dw, -dg);
-        else
-          dd[j] = fma(A, dw, dg);
-        if (j == 2) dw2 = dw;
+        dw[j] = pl[0][f + j + 1] - pl[0][f + j];
+        dg[j] = pl[1][f + j + 1] - pl[1][f + j];
+        xw[j] = __dmul_rn(A, dw[j]);
       }
-      base = fma(-A, dw2, pl[1][f + 2] + pl[1][f + 3]);
-      part = za6d<AI, P1>(dd[0], dd[1], dd[2], dd[3], dd[4], rp);
+      centre = pl[1][f + 2] + pl[1][f + 3];
+      es = fx::top_exponent(xw, dg);
     }
-    const ZA6Part other = {__shfl_xor_sync(0xffffffffu, part.num, 1),
-                           __shfl_xor_sync(0xffffffffu, part.den, 1)};
-    if (act && sgn == 0) fl[f][0] = pair_flux(base, part, other);
+    const bool fixed = P1 && act && es >= rp.es_lo && es <= rp.es_hi;
+    if (fixed) {
+      fx::i64 d[5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const fx::i64 x = fx::to_fixed(xw[j], es), g = fx::to_fixed(dg[j], es);
+        if (sgn)
+          d[4 - j] = x - g;
+        else
+          d[j] = x + g;
+      }
+      if constexpr (AI == kAiTiny)
+        c = fx::recon6<false>(d[0], d[1], d[2], d[3], d[4], rp.e3);
+      else
+        c = fx::recon6<true>(d[0], d[1], d[2], d[3], d[4], sens_fixed<AI>(d, es, rp));
+    }
+    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    if (act && sgn == 0) {
+      if (fixed)
+        fl[f][0] = __fma_rn((double)c, fx::scale_back(es), __dsub_rn(centre, xw[2]));
+      else
+        fl[f][0] = field_flux<AI, P1>(dw, dg, A, rp, centre);
+    }
   } else {
     const int f = tid;  // face between cells i0+f-1 and i0+f; stencil f..f+2R-1
     if (f <= T && i0 + f - 1 < nx) {
@@ -189,13 +207,13 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
           }
           h = field_flux_f32<P1>(w, g, A, s_r32);
         } else if constexpr (R == 3) {
-          double w[6], g[6];
+          double dw[5], dg[5];
 #pragma unroll
-          for (int j = 0; j < 6; ++j) {
-            w[j] = pl[0][f + j];
-            g[j] = pl[1][f + j];
+          for (int j = 0; j < 5; ++j) {
+            dw[j] = pl[0][f + j + 1] - pl[0][f + j];
+            dg[j] = pl[1][f + j + 1] - pl[1][f + j];
           }
-          h = field_flux<AI, P1>(w, g, A, s_rp[0]);
+          h = field_flux<AI, P1>(dw, dg, A, s_rp[0], pl[1][f + 2] + pl[1][f + 3]);
         } else {
           const ReconParams rp = s_rp[0];
           double pp[N], mm[N];  // f^+ in stencil order, f^- mirrored
@@ -232,9 +250,9 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
             h2 = field_flux_f32d<P1>(dW[1], dG[1], A2, s_r32);
             h3 = field_flux_f32d<P1>(dW[2], dG[2], A3, s_r32);
           } else {
-            h1 = field_flux_d<AI, P1>(dW[0], dG[0], A1, s_rp[1]);
-            h2 = field_flux_d<AI, P1>(dW[1], dG[1], A2, s_rp[0]);
-            h3 = field_flux_d<AI, P1>(dW[2], dG[2], A3, s_rp[1]);
+            h1 = field_flux<AI, P1>(dW[0], dG[0], A1, s_rp[1], 0.0);
+            h2 = field_flux<AI, P1>(dW[1], dG[1], A2, s_rp[0], 0.0);
+            h3 = field_flux<AI, P1>(dW[2], dG[2], A3, s_rp[1], 0.0);
           }
         } else {
           const ReconParams rp4 = s_rp[1], rp2 = s_rp[0];
@@ -310,7 +328,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
   }
 }
 
-template <int NC, bool AI, bool P1, int PREC, int R = 3>
+template <int NC, int AI, bool P1, int PREC, int R = 3>
 __global__ void __launch_bounds__(kThreads1D) k_line1d(const StageArgs a) {
   extern __shared__ double sm[];
   line1d_tile<NC, AI, P1, PREC, kT1, R>(a, blockIdx.y, blockIdx.x,
@@ -321,7 +339,7 @@ __global__ void __launch_bounds__(kThreads1D) k_line1d(const StageArgs a) {
 // (41 cells a tile) or 2 per face for a scalar (63 cells).
 __host__ __device__ constexpr int kT1Lanes(int nc) { return nc == 3 ? 41 : 63; }
 
-template <int NC, bool AI, bool P1, int PREC>
+template <int NC, int AI, bool P1, int PREC>
 __global__ void __launch_bounds__(kThreads1D) k_line1d_lanes(const StageArgs a) {
   extern __shared__ double sm[];
   line1d_tile<NC, AI, P1, PREC, kT1Lanes(NC), 3, (NC == 3 ? 3 : 2)>(

@@ -15,6 +15,7 @@
 //    sub-expressions, two of their rows and the 1/2 of eq. (6) folded into
 //    the back-projection.
 #pragma once
+#include <climits>
 #include <cstdint>
 
 #include "weno_fixed.cuh"
@@ -427,11 +428,11 @@ __device__ __noinline__ double pair_wide(double base, const double *dw, const do
                    za6d<(AI != kNoAi), P1>(dm[0], dm[1], dm[2], dm[3], dm[4], P));
 }
 
-// The sensitivity term of recon6 for one stencil (see there), in its units:
+// The sensitivity term of recon6 for one stencil (see there) in units of 2^k:
 // constant without the descaler, else 3 (sqrt(4 eps) mu)^2 from the mean
 // deviation of the stencil in FP64.
 template <int AI>
-__device__ __forceinline__ fx::Flt sens_fixed(const fx::i64 (&d)[5], int es,
+__device__ __forceinline__ fx::Flt sens_fixed(const fx::i64 (&d)[5], int k,
                                               const ReconParams &P) {
   fx::Flt e = P.e3;
   if constexpr (AI == kAi) {
@@ -441,29 +442,37 @@ __device__ __forceinline__ fx::Flt sens_fixed(const fx::i64 (&d)[5], int es,
     const double m = ((a0 + a1) + (a3 + a4) + a5) * (1.0 / 6.0);
     const double dev = fabs(a0 - m) + fabs(a1 - m) + fabs(m) + fabs(a3 - m) + fabs(a4 - m) +
                        fabs(a5 - m);
-    const double unit = __longlong_as_double((long long)(es - 56) << 52);  // 2^(es - 1079)
+    const double unit = __longlong_as_double((long long)(k + 1023) << 52);  // 2^k
     const double sm = fma(dev * unit, P.me, P.mo);
     const unsigned long long b = (unsigned long long)__double_as_longlong(3.0 * (sm * sm));
     e.m = (b << 11) | 0x8000000000000000ull;
     e.e = (int)(b >> 52) - 1086;
   }
-  e.e -= 2 * (es - 1079);
+  e.e -= 2 * k;
   return e;
 }
 
-// One characteristic field of one face (FP64) from the differences dw[j] =
-// w_{j+1} - w_j, dg[j] = g_{j+1} - g_j of its projected states and fluxes over
-// the six stencil cells; A is the field's GLF speed.  The split of eq. (6)
-// (kernel scaling: without the 1/2) is applied to the differences: f+ = g + A w
-// has differences dg + A dw, and the mirrored f- = g - A w, read from i+3 down
-// to i-2, has differences A dw - dg in reverse order.  Returns
-// h = f^+ + f^- at i+1/2 with centre = g_i + g_{i+1}, or h less those centre
-// values with centre = 0 (the Euler kernels add them back in physical form
-// after the back-projection, where R (g_i + g_{i+1}) is F_i + F_{i+1}).
+template <int AI>
+__device__ __forceinline__ fx::i64 recon_fixed(const fx::i64 (&d)[5], int k, const ReconParams &P) {
+  if constexpr (AI == kAiTiny)
+    return fx::recon6<false>(d[0], d[1], d[2], d[3], d[4], P.e3);
+  else
+    return fx::recon6<true>(d[0], d[1], d[2], d[3], d[4], sens_fixed<AI>(d, k, P));
+}
+
+// One field of one face (FP64) from the differences dw[j] = w_{j+1} - w_j,
+// dg[j] = g_{j+1} - g_j of its states and fluxes over the six stencil cells; A
+// is the field's GLF speed.  The split of eq. (6) (kernel scaling: without the
+// 1/2) is applied to the differences: f+ = g + A w has differences dg + A dw,
+// and the mirrored f- = g - A w, read from i+3 down to i-2, has differences
+// A dw - dg in reverse order.  Returns h = f^+ + f^- at i+1/2 with centre =
+// g_i + g_{i+1}, or h less those centre values with centre = 0.
 // For p = 1 the two reconstructions run on the integer pipes (recon6 in
-// weno_fixed.cuh) in units of the ten differences' largest exponent; what is
-// left to FP64 is A dw, the sum's conversion and its scaling: 7 operations a
-// field instead of 120.  A field that does not vary at all needs neither.
+// weno_fixed.cuh) in units of the ten differences' largest exponent, one after
+// the other in a loop (unrolled, the code of a face outgrows the instruction
+// cache); what is left to FP64 is A dw, the sum's conversion and its scaling:
+// 7 operations a field instead of 120.  A field that does not vary at all
+// needs neither.
 template <int AI, bool P1>
 __device__ __forceinline__ double field_flux(const double (&dw)[5], const double (&dg)[5],
                                              double A, const ReconParams &P, double centre) {
@@ -474,20 +483,19 @@ __device__ __forceinline__ double field_flux(const double (&dw)[5], const double
   if constexpr (P1) {
     const int es = fx::top_exponent(xw, dg);
     if (es >= P.es_lo && es <= P.es_hi) {
-      fx::i64 p[5], n[5];
+      fx::i64 x[5], g[5], c = 0;
 #pragma unroll
       for (int j = 0; j < 5; ++j) {
-        const fx::i64 x = fx::to_fixed(xw[j], es), g = fx::to_fixed(dg[j], es);
-        p[j] = x + g;
-        n[4 - j] = x - g;
+        x[j] = fx::to_fixed(xw[j], es);
+        g[j] = fx::to_fixed(dg[j], es);
       }
-      fx::i64 c;
-      if constexpr (AI == kAiTiny) {
-        c = fx::recon6<false>(p[0], p[1], p[2], p[3], p[4], P.e3) +
-            fx::recon6<false>(n[0], n[1], n[2], n[3], n[4], P.e3);
-      } else {
-        c = fx::recon6<true>(p[0], p[1], p[2], p[3], p[4], sens_fixed<AI>(p, es, P)) +
-            fx::recon6<true>(n[0], n[1], n[2], n[3], n[4], sens_fixed<AI>(n, es, P));
+#pragma unroll 1
+      for (int s = 0; s < 2; ++s) {
+        fx::i64 d[5];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) d[j] = x[j] + g[j];
+        c += recon_fixed<AI>(d, es - 1079, P);
+        fx::mirror(x, g);
       }
       return __fma_rn((double)c, fx::scale_back(es), base);
     }
@@ -1022,6 +1030,165 @@ __device__ __forceinline__ void backproject3(const FaceState &f, double h1, doub
   F0 = S;
   F1 = fma(f.un, S, f.c * D);
   F2 = fma(f.H, h13, fma(f.un * f.c, D, f.q2 * h2));
+}
+
+// Exponent codes of a face's five pairs (weno_fixed.cuh) with fluxes aligned
+// to 2^a times the states: false if a difference is outside the packed range.
+template <int NC, class DU, class DF>
+__device__ __forceinline__ bool face_exponents(int a, DU du, DF df, int (&E)[NC]) {
+  int top = 0;
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    int eu = 0, ef = 0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      eu = max(eu, fx::packed_exponent(du(q, j)));
+      ef = max(ef, fx::packed_exponent(df(q, j)));
+    }
+    top = max(top, max(eu, ef));
+    E[q] = max(eu, ef - a);
+  }
+  return top < fx::kWide;
+}
+
+// c^+ + c^- less 6 alpha dw_2 of one field (weno_fixed.cuh) from its projected
+// differences w of the states and g of the fluxes in units of 2^k0, and the
+// speed A; k is the scale of the result, or INT_MIN where the field is left
+// to FP64.  Calls, so that their code is there once: inlined for every field,
+// a face's code outgrows the instruction cache.
+struct FieldSum {
+  fx::i64 S;
+  int k;
+};
+template <int AI>
+__device__ __noinline__ fx::i64 rough_call(fx::i64 x0, fx::i64 x1, fx::i64 x2, fx::i64 x3,
+                                           fx::i64 x4, fx::i64 g0, fx::i64 g1, fx::i64 g2,
+                                           fx::i64 g3, fx::i64 g4, int k, const ReconParams &P) {
+  fx::i64 x[5] = {x0, x1, x2, x3, x4}, g[5] = {g0, g1, g2, g3, g4};
+  return fx::rough_sum(x, g, [&](const fx::i64(&d)[5]) { return recon_fixed<AI>(d, k, P); });
+}
+__device__ __forceinline__ bool in_range(int k, const ReconParams &P) {
+  const int es = k + 1080;
+  return es >= P.es_lo && es <= P.es_hi;
+}
+template <int AI>
+__device__ __noinline__ FieldSum field_call(fx::i64 w0, fx::i64 w1, fx::i64 w2, fx::i64 w3,
+                                            fx::i64 w4, fx::i64 g0, fx::i64 g1, fx::i64 g2,
+                                            fx::i64 g3, fx::i64 g4, fx::Limb A, int k0,
+                                            const ReconParams &P) {
+  fx::i64 x[5] = {w0, w1, w2, w3, w4}, g[5] = {g0, g1, g2, g3, g4};
+#pragma unroll
+  for (int j = 0; j < 5; ++j) x[j] = fx::times_speed(A, x[j]);
+  const int n = fx::field_shift(x, g);
+  if (n == 64) return FieldSum{0, 0};
+  const int k = k0 + 6 - n;
+  if (!in_range(k, P)) return FieldSum{0, INT_MIN};
+  fx::shift_field(x, n);
+  fx::shift_field(g, n);
+  int cp = 0, cm = 0;
+  bool smooth = true;
+#pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+    fx::i64 d[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) d[j] = x[j] + g[j];
+    smooth = fx::smooth_term<(AI != kAiTiny)>(d, cm) && smooth;
+    cp += cm;
+    fx::mirror(x, g);
+  }
+  return FieldSum{smooth ? fx::smooth_sum(g, cp)
+                         : rough_call<AI>(x[0], x[1], x[2], x[3], x[4], g[0], g[1], g[2], g[3],
+                                          g[4], k, P),
+                  k};
+}
+// h of one field less its centre values; wide() gives it in FP64 where ok is
+// false or field_call leaves it.
+template <int AI, class Wide>
+__device__ __forceinline__ double field_fixed(const fx::i64 (&w)[5], const fx::i64 (&g)[5],
+                                              const fx::Limb &A, int k0, bool ok,
+                                              const ReconParams &P, Wide wide) {
+  const FieldSum s = field_call<AI>(w[0], w[1], w[2], w[3], w[4], g[0], g[1], g[2], g[3], g[4],
+                                    A, k0, P);
+  if (!ok || s.k == INT_MIN) return wide();
+  return (double)s.S * fx::sixth(s.k);
+}
+
+__device__ __forceinline__ fx::i64 shfl64(fx::i64 v, int src) {
+  return __shfl_sync(0xffffffffu, v, src);
+}
+// The same spread over two lanes of a warp (every lane of the warp calls this):
+// lane sgn = 0 brings the projected state differences, lane sgn = 1 those of
+// the flux, `other` is the partner; each reconstructs one of the fluxes.  The
+// operations are field_call's.  Returns h on both lanes, wide = true where
+// the field is left to FP64.
+template <int AI>
+__device__ __forceinline__ double field_lanes(const fx::i64 (&v)[5], const fx::Limb &A, int k0,
+                                              bool ok, int sgn, int other, const ReconParams &P,
+                                              bool &wide) {
+  fx::i64 x[5], g[5];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const fx::i64 own = sgn ? v[j] : fx::times_speed(A, v[j]), got = shfl64(own, other);
+    x[j] = sgn ? got : own;
+    g[j] = sgn ? own : got;
+  }
+  const int n = fx::field_shift(x, g), k = n == 64 ? 0 : k0 + 6 - n;
+  wide = !ok || (n < 64 && !in_range(k, P));
+  fx::shift_field(x, n == 64 ? 1 : n);
+  fx::shift_field(g, n == 64 ? 1 : n);
+  if (sgn) fx::mirror(x, g);
+  fx::i64 d[5];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) d[j] = x[j] + g[j];
+  int c;
+  const bool own = fx::smooth_term<(AI != kAiTiny)>(d, c);
+  const int c2 = __shfl_sync(0xffffffffu, own ? c : INT_MIN, other);
+  const bool smooth = own && c2 != INT_MIN;
+  fx::i64 r = 0;
+  if (!smooth && !wide && n < 64) r = recon_fixed<AI>(d, k, P) - 3 * d[2];
+  r += shfl64(r, other);
+  if (sgn) fx::mirror(x, g);
+  const fx::i64 S = smooth ? fx::smooth_sum(g, c + c2) : r;
+  return n == 64 ? 0.0 : (double)S * fx::sixth(k);
+}
+
+// The fields of one face from its packed differences du(q, j), df(q, j) of
+// states and physical fluxes, component q, pair j; KA[m] and a: the fields'
+// speeds (fx::speed).
+template <int NC, int AI, class DU, class DF, class Wide, class RP>
+__device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb *KA, int a, DU du,
+                                            DF df, RP rp, Wide wide, double (&h)[NC]) {
+  int E[NC];
+  bool ok = face_exponents<NC>(a, du, df, E);
+  const fx::LeftRows<NC> rows =
+      fx::left_rows<NC>(E, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic), __dmul_rn(fs.b1, fs.un),
+                        __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
+  ok = ok && rows.emax < 2047;
+  fx::Proj U[5], F[5];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    fx::u64 v[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) v[q] = du(q, j);
+    U[j] = fx::project<NC>(rows, E, 0, v);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) v[q] = df(q, j);
+    F[j] = fx::project<NC>(rows, E, a, v);
+  }
+  const int k0 = rows.um + a - 1592;
+  auto field = [&](int m, int k, auto part) {
+    fx::i64 w[5], g[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      w[j] = part(U[j]);
+      g[j] = part(F[j]);
+    }
+    h[m] = field_fixed<AI>(w, g, KA[m], k, ok, rp(m), [&]() { return wide(m); });
+  };
+  if constexpr (NC == 4) field(2, rows.us + a - 1592, [](const fx::Proj &p) { return p.s; });
+  field(1, k0, [](const fx::Proj &p) { return p.r - p.z; });
+  field(0, k0, [](const fx::Proj &p) { return p.z + p.tc; });
+  field(NC - 1, k0, [](const fx::Proj &p) { return p.z - p.tc; });
 }
 
 }  // namespace weno

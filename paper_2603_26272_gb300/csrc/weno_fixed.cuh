@@ -245,5 +245,278 @@ WENO_FX double scale_back(int es) {
   return bitsd(dbits(1.0 / 6.0) + ((u64)(i64)(es - 1079) << 52));
 }
 
+// ---------------------------------------------------------------------------
+// Projection on the face's left eigenvectors, on the integer pipes.
+//
+// The kernels stage differences between adjacent cells packed in 64 bits: the
+// signed 53-bit mantissa of the double above a 10-bit exponent code (0: the
+// value is 0; kWide: not finite, or not 0 and outside 2^-511 .. 2^511, which
+// the integer path leaves to FP64), so a face aligns one with a mask and a
+// shift.  Per face and component q the exponent E_q is the largest of the
+// stencil's five pairs; the eigenvectors' coefficients get the scale that
+// brings the largest coefficient times its component below 2^61 both ways, and
+// a coefficient times a component is a 64 x 64-bit product of 32-bit limbs, three
+// multiply-adds.
+// ---------------------------------------------------------------------------
+constexpr int kWide = 1023;
+WENO_FX u64 pack(double x) {
+  const u64 b = dbits(x);
+  const int e = (int)((b >> 52) & 0x7FF);
+  const u64 m = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  const bool in = e >= 512 && e <= 1533, zero = (b << 1) == 0;
+  return zero ? 0 : ((((i64)b < 0 ? 0 - m : m) << 10) | (u64)(in ? e - 511 : kWide));
+}
+WENO_FX int packed_exponent(u64 w) { return (int)(w & 0x3FF); }
+// Sign-extending shift of the packed mantissa; a count of 64 or more leaves
+// the sign.
+WENO_FX i64 packed_value(u64 w, int n) {
+  const i64 v = (i64)(w & ~0x3FFull);
+#ifdef __CUDA_ARCH__
+  i64 r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return v >> (n > 63 ? 63 : n);
+#endif
+}
+
+// A number as two limbs, 2^32 h + 2 l (its lowest bit dropped): all products
+// of limbs are signed 32 x 32 -> 64 bits.
+struct Limb {
+  int h, l;
+};
+WENO_FX Limb limb(i64 v) {
+  Limb o;
+  o.h = (int)(v >> 32);
+  o.l = (int)(lo32((u64)v) >> 1);
+  return o;
+}
+// Sum of products in units of 2^64 (hi) and 2^33 (cr): of four with factors
+// below 2^61 (the products of the low limbs, left out, are then a relative
+// 2^-58).
+struct Acc {
+  i64 hi, cr;
+};
+WENO_FX i64 acc_value(const Acc &a) { return (a.hi << 1) + (a.cr >> 30); }  // sum / 2^63
+WENO_FX void mac(Acc &s, const Limb &a, const Limb &b) {
+  s.hi += (i64)a.h * b.h;
+  s.cr += (i64)a.h * b.l;
+  s.cr += (i64)a.l * b.h;
+}
+
+// The integer form of a coefficient: x 2^(1083 + E - um) with E an exponent
+// code (|result| < 2^61 for um >= exponent(x) + E).
+WENO_FX Limb coefficient(double x, int E, int um) {
+  const u64 b = dbits(x);
+  const int e = (int)((b >> 52) & 0x7FF);
+  const u64 m = e ? (b << 11) | 0x8000000000000000ull : 0;
+  const u64 v = shr(m, um - e - E + 3);
+  return limb((i64)b < 0 ? -(i64)v : (i64)v);
+}
+WENO_FX int exponent(double x) { return (int)((hi32(dbits(x)) >> 20) & 0x7FF); }
+WENO_FX int imax(int a, int b) { return a > b ? a : b; }
+// A GLF speed A < 2^a as A 2^(63 - a).
+WENO_FX Limb speed(double A, int a) {
+  const u64 b = dbits(A);
+  const int e = (int)(b >> 52);
+  return limb((i64)shr(e ? (b << 11) | 0x8000000000000000ull : 0, a + 1023 - e));
+}
+// A w / 2^a for |w| < 2^62.
+WENO_FX i64 times_speed(const Limb &A, i64 w) {
+  Acc v = {0, 0};
+  mac(v, A, limb(w));
+  return acc_value(v);
+}
+
+// The left eigenvectors of a face in the form project4 (NC = 4) and project3
+// (NC = 3) apply them: with z = b2 r - t2 m_n - t3 m_t + b1 E and
+// tc = t1 r - ic m_n the fields are z + tc, r - z, (m_t - ut r,) z - tc.
+// um: the scale of z, tc and r, projected values are x 2^(1592 - um) (below
+// 2^61.6); ut: that of m_t - ut r.  emax: the largest exponent among the
+// coefficients (2047: not finite).
+template <int NC>
+struct LeftRows {
+  Limb zr, zn, zt, zE, tr, tn, sr;
+  int um, us, emax;
+};
+template <int NC>
+WENO_FX LeftRows<NC> left_rows(const int (&E)[NC], double b2, double b1, double t1, double t2,
+                               double t3, double ic, double ut) {
+  LeftRows<NC> o;
+  const int e1 = exponent(b1), e2 = exponent(b2), f1 = exponent(t1), f2 = exponent(t2),
+            f3 = exponent(t3), fc = exponent(ic), fu = exponent(ut);
+  o.emax = imax(imax(imax(e1, e2), imax(f1, f2)), imax(fc, NC == 4 ? imax(f3, fu) : 0));
+  o.um = imax(imax(imax(e2, f1), 1023) + E[0], imax(imax(f2, fc) + E[1], e1 + E[NC - 1]));
+  o.us = 0;
+  if (NC == 4) {
+    o.um = imax(o.um, f3 + E[2]);
+    o.us = imax(fu + E[0], 1023 + E[2]);
+    o.zt = coefficient(-t3, E[2], o.um);
+    o.sr = coefficient(-ut, E[0], o.us);
+  }
+  o.zr = coefficient(b2, E[0], o.um);
+  o.zn = coefficient(-t2, E[1], o.um);
+  o.zE = coefficient(b1, E[NC - 1], o.um);
+  o.tr = coefficient(t1, E[0], o.um);
+  o.tn = coefficient(-ic, E[1], o.um);
+  return o;
+}
+// A difference vector's projections: z, tc, r (and s = m_t - ut r) from its
+// packed components v[q], with a = 0 for states, the speeds' exponent for
+// physical fluxes.
+struct Proj {
+  i64 z, tc, r, s;
+};
+template <int NC>
+WENO_FX Proj project(const LeftRows<NC> &c, const int (&E)[NC], int a, const u64 (&v)[NC]) {
+  Limb d[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) d[q] = limb(packed_value(v[q], E[q] + a + 2 - packed_exponent(v[q])));
+  Acc z = {0, 0}, t = {0, 0};
+  mac(z, c.zr, d[0]);
+  mac(z, c.zn, d[1]);
+  if (NC == 4) mac(z, c.zt, d[2]);
+  mac(z, c.zE, d[NC - 1]);
+  mac(t, c.tr, d[0]);
+  mac(t, c.tn, d[1]);
+  Proj o;
+  o.z = acc_value(z);
+  o.tc = acc_value(t);
+  o.r = packed_value(v[0], c.um + a - 1018 - packed_exponent(v[0]));
+  o.s = 0;
+  if (NC == 4) {
+    Acc u = {0, 0};
+    mac(u, c.sr, d[0]);
+    o.s = acc_value(u) + packed_value(v[2], c.us + a - 1018 - packed_exponent(v[2]));
+  }
+  return o;
+}
+
+// The stencil differences g + x of f^+ become those of the mirrored f^-:
+// x - g in reverse order.
+WENO_FX void mirror(i64 (&x)[5], i64 (&g)[5]) {
+  const i64 x0 = x[0], x1 = x[1], g0 = g[0], g1 = g[1];
+  x[0] = x[4];
+  x[4] = x0;
+  x[1] = x[3];
+  x[3] = x1;
+  g[0] = -g[4];
+  g[4] = -g0;
+  g[1] = -g[3];
+  g[3] = -g1;
+  g[2] = -g[2];
+}
+
+// Shift of a field's differences that brings the largest |g +- x| to
+// [2^57, 2^58): left by n - 6 (n = 64: they are all 0).
+WENO_FX int field_shift(const i64 (&x)[5], const i64 (&g)[5]) {
+  uint32_t mh = 0, ml = 0;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const i64 p = x[j] + g[j], n = x[j] - g[j], sp = p >> 63, sn = n >> 63;
+    mh |= hi32((u64)(p ^ sp)) | hi32((u64)(n ^ sn));
+    ml |= lo32((u64)(p ^ sp)) | lo32((u64)(n ^ sn));
+  }
+  return clz64(((u64)mh << 32) | ml);
+}
+WENO_FX void shift_field(i64 (&x)[5], int n) {
+#pragma unroll
+  for (int j = 0; j < 5; ++j) x[j] = (i64)shl((u64)x[j], n - 1) >> 5;
+}
+
+// FP32 operations that no compiler contracts: every kernel takes the same
+// decision, and the same term, for the same stencil.
+#ifdef __CUDA_ARCH__
+WENO_FX float fmul(float a, float b) { return __fmul_rn(a, b); }
+WENO_FX float fadd(float a, float b) { return __fadd_rn(a, b); }
+WENO_FX float ffma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+#else
+WENO_FX float fmul(float a, float b) { return a * b; }
+WENO_FX float fadd(float a, float b) { return a + b; }
+WENO_FX float ffma(float a, float b, float c) { return std::fma(a, b, c); }
+#endif
+// A 64-bit integer over 2^32 in FP32.
+WENO_FX float to_float(i64 x) {
+  return ffma((float)lo32((u64)x), 0x1p-32f, (float)(int)hi32((u64)x));
+}
+WENO_FX float rcpf(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return 1.0f / x;
+#endif
+}
+
+// Smooth stencils.  With the linear candidate average rm = sum D_k r_k / 20,
+//   c = rm + sum_k D_k G_k (r_k - rm) / (20 + sum_k D_k G_k), G_k = T / b_k,
+// the second term is far below a unit, or a few units, wherever the stencil
+// resolves its data (G is the eighth power of the phase per cell, r_k - rm its
+// third): computed in FP32 on the exact second and fifth differences, with an
+// error below 2^-21 of max G max |r_k - rm|, it is good to half a unit where
+// that product is at most 2^20 units, from about 70 cells a wavelength on.
+// Returns whether it is, and the term in units.
+// SENS: a sensitivity term would lower G; the term then has to vanish (at
+// most half a unit).
+template <bool SENS>
+WENO_FX bool smooth_term(const i64 (&d)[5], int &corr) {
+  const i64 s0 = d[1] - d[0], s1 = d[2] - d[1], s2 = d[3] - d[2], s3 = d[4] - d[3];
+  const i64 q = s1 - s2;
+  const float r5 = to_float((s3 - s0) + 3 * q);
+  const float a0 = to_float(s0), a1 = to_float(s1), a2 = to_float(s2), a3 = to_float(s3);
+  const float f1 = to_float(d[1]), f2 = to_float(d[2]), f3 = to_float(d[3]);
+  const float t0 = ffma(2.0f, f1, a0), t1 = fadd(f1, f2), t2 = ffma(2.0f, f2, -a2),
+              t3 = ffma(3.0f, a3, fmul(-2.0f, f3));
+  const float b0 = ffma(fmul(13.0f, a0), a0, fmul(fmul(3.0f, t0), t0));
+  const float b1 = ffma(fmul(13.0f, a1), a1, fmul(fmul(3.0f, t1), t1));
+  const float b2 = ffma(fmul(13.0f, a2), a2, fmul(fmul(3.0f, t2), t2));
+  const float bd = ffma(fmul(13.0f, a3), a3, fmul(fmul(3.0f, t3), t3));
+  const float b3 = fmul(0.25f, fadd(fadd(b0, b1), fadd(b2, bd)));
+  const float T = fmul(fmul(12.0f, r5), r5), T9 = fmul(9.0f, T), tiny = 1e-30f;
+  const float g0 = fmul(T, rcpf(fadd(b0, tiny))), g1 = fmul(T9, rcpf(fadd(b1, tiny)));
+  const float g2 = fmul(T9, rcpf(fadd(b2, tiny))), g3 = fmul(T, rcpf(fadd(b3, tiny)));
+  // r_k - r_1, their mean m, and r_k - rm
+  const float e0 = fmul(2.0f, to_float(s0 - s1)), e2 = to_float(q);
+  const float e3 = ffma(2.0f, to_float(s3 - s2), e2);
+  const float m = fmul(0.05f, ffma(9.0f, e2, fadd(e0, e3)));
+  const float h0 = fadd(e0, -m), h2 = fadd(e2, -m), h3 = fadd(e3, -m);
+  const float gs = fadd(fadd(g0, g1), fadd(g2, g3));  // 20 times a mean of the G_k
+  const float hm = fmaxf(fmaxf(fabsf(h0), fabsf(h2)), fmaxf(fabsf(h3), fabsf(m)));
+  const float c = fmul(ffma(g0, h0, ffma(g2, h2, ffma(g3, h3, -fmul(g1, m)))),
+                       rcpf(fadd(20.0f, gs)));
+  const bool ok = fmul(gs, hm) <= (SENS ? 8 * 0x1p-32f : 16 * 0x1p-12f);
+  corr = (SENS || !ok) ? 0 : (int)ffma(c, 0x1p32f, c < 0.0f ? -0.5f : 0.5f);
+  return ok;
+}
+
+// c^+ + c^- less 6 alpha dw_2 of a smooth field: the linear parts add up to
+// (7 (g_1 - g_3) - (g_0 - g_4)) / 5 (alpha drops out of the central flux).
+WENO_FX i64 smooth_sum(const i64 (&g)[5], int corr) {
+  const i64 v = 7 * (g[1] - g[3]) - (g[0] - g[4]);  // below 2^63
+  // v / 5 = (v >> 32) 2^32 / 5 + ..: 2^63 / 5 in two limbs
+  Acc p = {0, 0};
+  mac(p, Limb{0x19999999, 0x4CCCCCCD}, limb(v));
+  return (p.hi << 1) + (p.cr >> 30) + corr;
+}
+
+// c^+ + c^- less 6 alpha dw_2 by the weights, one flux after the other.
+template <class Recon>
+WENO_FX i64 rough_sum(i64 (&x)[5], i64 (&g)[5], Recon recon) {
+  i64 S = 0;
+#pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+    i64 d[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) d[j] = x[j] + g[j];
+    S += recon(d) - 3 * d[2];
+    mirror(x, g);
+  }
+  return S;
+}
+
+// 2^k / 6 for -1019 <= k <= 1026.
+WENO_FX double sixth(int k) { return bitsd(dbits(1.0 / 6.0) + ((u64)(i64)k << 52)); }
+
 }  // namespace fx
 }  // namespace weno

@@ -604,137 +604,204 @@ __device__ __forceinline__ void normal_flux(double rho, double mn, double mt, do
   F3 = H * mn;
 }
 
-template <int TX, int TY, int AI, bool P1, int PREC, int DIR>
-__device__ __forceinline__ void tile6_sweep(const StageArgs &a, long long b, long long i0,
+// GLF speed of field m of nc (max|u| + c for every field in the single mode).
+__device__ __forceinline__ double field_speed(const StageArgs &a, const unsigned long long *al,
+                                              int m, int nc) {
+  unsigned long long v = al[m];
+  if (a.alpha_single)
+    for (int q = 0; q < nc; ++q) v = max(v, al[q]);
+  return bits2d(v);
+}
+
+// The GLF speeds of a problem in fixed point, per direction (fx::speed), and
+// the exponents above them; the block's first threads form them once.
+struct Speeds {
+  fx::Limb ka[2][4];
+  int ea[2];
+};
+__device__ __forceinline__ void make_speeds(const StageArgs &a, long long b, int nc, Speeds &s) {
+  const int dir = threadIdx.x >> 2, m = threadIdx.x & 3;
+  if (dir >= a.ndim || m >= nc) return;
+  const unsigned long long *al = a.alpha_in + b * 8 + 4 * dir;
+  unsigned long long top = al[0];
+  for (int q = 1; q < nc; ++q) top = max(top, al[q]);
+  const int ea = fx::exponent(bits2d(top)) - 1022;
+  s.ka[dir][m] = fx::speed(field_speed(a, al, m, nc), ea);
+  if (m == 0) s.ea[dir] = ea;
+}
+
+// Field m of face (fr, fc) along DIR in FP64 from the staged cells (less its
+// centre values): what the integer path leaves out.
+template <int TX, int TY, int AI>
+__device__ __noinline__ double face_wide(const double *sm, int dir, int fr, int fc, int m, double un,
+                                         double ut, double ic, double b1, double b2, double A,
+                                         const ReconParams &rp) {
+  using L = Tile6<TX, TY>;
+  const double *const box = sm + L::kBox, *const pl = sm + L::kPl;
+  FaceState fs = {};
+  fs.un = un;
+  fs.ut = ut;
+  fs.ic = ic;
+  fs.b1 = b1;
+  fs.b2 = b2;
+  double U[2][4], F[2][4], dw[5], dg[5];
+  for (int j = 0; j < 6; ++j) {
+    const int r = dir ? fr + j : 3 + fr, c = dir ? 3 + fc : fc + j;
+    const int o = r * L::BW + c + L::XO - 3, k = r * L::W + c;
+    double *const u = U[j & 1], *const f = F[j & 1];
+    u[0] = box[o];
+    u[1] = f[0] = box[(1 + dir) * L::PB + o];
+    u[2] = box[(2 - dir) * L::PB + o];
+    u[3] = box[3 * L::PB + o];
+    normal_flux(u[0], u[1], u[2], u[3], pl[(1 + dir) * L::REG + k], pl[3 * L::REG + k], f[1], f[2],
+                f[3]);
+    if (j == 0) continue;
+    const double *const u0 = U[(j - 1) & 1], *const f0 = F[(j - 1) & 1];
+    double w[4], g[4];
+    project4(fs, u[0] - u0[0], u[1] - u0[1], u[2] - u0[2], u[3] - u0[3], w[0], w[1], w[2], w[3]);
+    project4(fs, f[0] - f0[0], f[1] - f0[1], f[2] - f0[2], f[3] - f0[3], g[0], g[1], g[2], g[3]);
+    dw[j - 1] = w[m];
+    dg[j - 1] = g[m];
+  }
+  return pair_wide<AI, true>(-A * dw[2], dw, dg, A, rp);
+}
+
+// One direction (0: x, 1: y) of a tile.  The direction is a run-time value: the
+// two sweeps then share their code, which has to stay in the instruction
+// cache.
+template <int TX, int TY, int AI, bool P1, int PREC>
+__device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long long b, long long i0,
                                             long long j0, double gm1, double *sm,
-                                            const ReconParams &rp2, const ReconParams &rp4) {
+                                            const ReconParams &rp2, const ReconParams &rp4,
+                                            const Speeds &sp) {
   using L = Tile6<TX, TY>;
   constexpr int R = 3, W = L::W, BW = L::BW, XO = L::XO, PB = L::PB, REG = L::REG, ND = L::ND;
   const double *const box = sm + L::kBox;
   const double *const pl = sm + L::kPl;
   double *const dd = sm + L::kDd;
-  double *const fo = sm + (DIR ? L::kFy : L::kFx);
+  double *const fo = sm + (dir ? L::kFy : L::kFx);
+  // p = 1 in FP64: packed differences, projected on the integer pipes
+  constexpr bool kPacked = P1 && PREC == 0;
+  fx::u64 *const dp = reinterpret_cast<fx::u64 *>(dd);
   const int tid = threadIdx.x;
-  // box offset of staged cell (r, c)
+  // offsets of staged cell (r, c) in the box and the planes, and to the next
+  // cell along the direction; planes of the normal and tangential momentum
+  // and velocity
   auto bo = [](int r, int c) { return r * BW + c + XO - R; };
+  const int stB = dir ? BW : 1, stP = dir ? W : 1;
+  const double *const bn = box + (1 + dir) * PB, *const bt = box + (2 - dir) * PB;
+  const double *const un = pl + (1 + dir) * REG, *const ut = pl + (2 - dir) * REG;
+  // k / d for the row lengths of pairs and faces (d <= 64, k < 1024)
+  auto rows_of = [](int k, int inv) { return (k * inv) >> 16; };
+  constexpr auto inv = [](int d) constexpr { return (65536 + d - 1) / d; };
 
-  // 1d: differences of each cell pair along DIR (normal frame: m_n = rho u
+  // 1d: differences of each cell pair along dir (normal frame: m_n = rho u
   // for x, rho v for y), in dd[q * ND + pair]:
   //   x: pair (rr, pc), rr in [0, TY), pc in [0, W - 1): cells (R + rr, pc), (R + rr, pc + 1)
   //   y: pair (pr, cc), pr in [0, HH - 1), cc in [0, TX): cells (pr, R + cc), (pr + 1, R + cc)
-  constexpr int NP = DIR ? L::NPY : L::NPX;
+  const int NP = dir ? L::NPY : L::NPX, lp = dir ? TX : W - 1, ip = dir ? inv(TX) : inv(W - 1);
   // the x pairs run from the block's last warp down: with phase 1 and the y
   // pairs starting from warp 0, the partial rounds of the three loops fall
   // on different warps (each warp's FP64 work goes to its own sub-partition)
-  const int t0 = DIR ? tid : (int)blockDim.x - 1 - tid;
-  for (int k = t0; k < NP; k += blockDim.x) {
-    int rA, cA, rB, cB;
-    if (DIR == 0) {
-      rA = R + k / (W - 1);
-      cA = k - (rA - R) * (W - 1);
-      rB = rA;
-      cB = cA + 1;
-    } else {
-      rA = k / TX;
-      cA = R + (k - rA * TX);
-      rB = rA + 1;
-      cB = cA;
-    }
-    const int oA = bo(rA, cA), oB = bo(rB, cB), kA = rA * W + cA, kB = rB * W + cB;
-    const double rhoA = box[oA], mnA = box[(1 + DIR) * PB + oA], mtA = box[(2 - DIR) * PB + oA],
-                 EA = box[3 * PB + oA];
-    const double rhoB = box[oB], mnB = box[(1 + DIR) * PB + oB], mtB = box[(2 - DIR) * PB + oB],
-                 EB = box[3 * PB + oB];
+  for (int k = dir ? tid : (int)blockDim.x - 1 - tid; k < NP; k += blockDim.x) {
+    const int q0 = rows_of(k, ip), q1 = k - q0 * lp;
+    const int rA = q0 + (dir ? 0 : R), cA = q1 + (dir ? R : 0);
+    const int oA = bo(rA, cA), oB = oA + stB, kA = rA * W + cA, kB = kA + stP;
+    const double rhoA = box[oA], mnA = bn[oA], mtA = bt[oA], EA = box[3 * PB + oA];
+    const double rhoB = box[oB], mnB = bn[oB], mtB = bt[oB], EB = box[3 * PB + oB];
     double F1A, F2A, F3A, F1B, F2B, F3B;
-    normal_flux(rhoA, mnA, mtA, EA, pl[(1 + DIR) * REG + kA], pl[3 * REG + kA], F1A, F2A, F3A);
-    normal_flux(rhoB, mnB, mtB, EB, pl[(1 + DIR) * REG + kB], pl[3 * REG + kB], F1B, F2B, F3B);
-    dd[0 * ND + k] = rhoB - rhoA;
-    dd[1 * ND + k] = mnB - mnA;  // also dF0
-    dd[2 * ND + k] = mtB - mtA;
-    dd[3 * ND + k] = EB - EA;
-    dd[4 * ND + k] = F1B - F1A;
-    dd[5 * ND + k] = F2B - F2A;
-    dd[6 * ND + k] = F3B - F3A;
+    normal_flux(rhoA, mnA, mtA, EA, un[kA], pl[3 * REG + kA], F1A, F2A, F3A);
+    normal_flux(rhoB, mnB, mtB, EB, un[kB], pl[3 * REG + kB], F1B, F2B, F3B);
+    const double d[7] = {rhoB - rhoA, mnB - mnA /* also dF0 */, mtB - mtA, EB - EA,
+                         F1B - F1A,   F2B - F2A,                F3B - F3A};
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      if constexpr (kPacked)
+        dp[q * ND + k] = fx::pack(d[q]);
+      else
+        dd[q * ND + k] = d[q];
+    }
   }
   __syncthreads();
 
-  // 2d: the faces along DIR.  x-face (fr, fc): between cells (R + fr, R - 1 + fc)
+  // 2d: the faces along dir.  x-face (fr, fc): between cells (R + fr, R - 1 + fc)
   // and (R + fr, R + fc), stencil pairs fr (W - 1) + fc + j; y-face (fr, fc):
   // between (R - 1 + fr, R + fc) and (R + fr, R + fc), pairs (fr + j) TX + fc.
-  constexpr int NF = DIR ? L::NFY : L::NFX;
-  const unsigned long long *al = a.alpha_in + b * 8 + 4 * DIR;
-  double A1 = bits2d(al[0]), A2 = bits2d(al[1]), A3 = bits2d(al[2]), A4 = bits2d(al[3]);
-  if (a.alpha_single) {
-    const double m = fmax(fmax(A1, A2), fmax(A3, A4));
-    A1 = A2 = A3 = A4 = m;
-  }
+  const int NF = dir ? L::NFY : L::NFX, lf = dir ? TX : TX + 1, jf = dir ? inv(TX) : inv(TX + 1);
+  const int ps = dir ? TX : 1;  // pair stride along the stencil
+  const unsigned long long *al = a.alpha_in + b * 8 + 4 * dir;
   const Recon32 r32 = make_r32(a);
   for (int f = tid; f < NF; f += blockDim.x) {
-    int fr, fc, p0, rL, cL, rR, cR;
-    constexpr int PS = DIR ? TX : 1;  // pair stride along the stencil
-    if (DIR == 0) {
-      fr = f / (TX + 1);
-      fc = f - fr * (TX + 1);
-      p0 = fr * (W - 1) + fc;
-      rL = R + fr;
-      cL = R - 1 + fc;
-      rR = rL;
-      cR = cL + 1;
-    } else {
-      fr = f / TX;
-      fc = f - fr * TX;
-      p0 = fr * TX + fc;
-      rL = R - 1 + fr;
-      cL = R + fc;
-      rR = rL + 1;
-      cR = cL;
-    }
-    const int kL = rL * W + cL, kR = rR * W + cR;
+    const int fr = rows_of(f, jf), fc = f - fr * lf;
+    const int p0 = fr * lp + fc;
+    const int rL = fr + (dir ? R - 1 : R), cL = fc + (dir ? R : R - 1);
+    const int kL = rL * W + cL, kR = kL + stP;
+    const int oL = bo(rL, cL), oR = oL + stB;
     FaceState fs;
-    if (!roe_face(pl[kL], pl[(1 + DIR) * REG + kL], pl[(2 - DIR) * REG + kL], pl[3 * REG + kL],
-                  pl[kR], pl[(1 + DIR) * REG + kR], pl[(2 - DIR) * REG + kR], pl[3 * REG + kR],
-                  gm1, fs))
+    if (!roe_face(pl[kL], un[kL], ut[kL], pl[3 * REG + kL], pl[kR], un[kR], ut[kR],
+                  pl[3 * REG + kR], gm1, fs))
       record_status(a.status, 3, a.stage, b, j0 + fr, i0 + fc);
-    double dw[4][5], dg[4][5];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      const int pj = p0 + j * PS;
-      const double dmn = dd[ND + pj];
-      project4(fs, dd[pj], dmn, dd[2 * ND + pj], dd[3 * ND + pj], dw[0][j], dw[1][j], dw[2][j],
-               dw[3][j]);
-      project4(fs, dmn, dd[4 * ND + pj], dd[5 * ND + pj], dd[6 * ND + pj], dg[0][j], dg[1][j],
-               dg[2][j], dg[3][j]);
-    }
-    double h1, h2, h3, h4;
-    if constexpr (PREC == 1) {
-      h1 = field_flux_f32d<P1>(dw[0], dg[0], A1, r32);
-      h2 = field_flux_f32d<P1>(dw[1], dg[1], A2, r32);
-      h3 = field_flux_f32d<P1>(dw[2], dg[2], A3, r32);
-      h4 = field_flux_f32d<P1>(dw[3], dg[3], A4, r32);
+    double h[4];
+    if constexpr (kPacked) {
+      const fx::u64 *const pf = dp + p0;
+      face_fields<4, AI>(
+          fs, sp.ka[dir], sp.ea[dir], [&](int q, int j) { return pf[q * ND + j * ps]; },
+          [&](int q, int j) { return pf[(q == 0 ? 1 : 3 + q) * ND + j * ps]; },
+          [&](int m) -> const ReconParams & { return (m == 0 || m == 3) ? rp4 : rp2; },
+          [&](int m) {
+            return face_wide<TX, TY, AI>(sm, dir, fr, fc, m, fs.un, fs.ut, fs.ic, fs.b1, fs.b2,
+                                         field_speed(a, al, m, 4), (m == 0 || m == 3) ? rp4 : rp2);
+          },
+          h);
     } else {
-      h1 = field_flux<AI, P1>(dw[0], dg[0], A1, rp4, 0.0);
-      h2 = field_flux<AI, P1>(dw[1], dg[1], A2, rp2, 0.0);
-      h3 = field_flux<AI, P1>(dw[2], dg[2], A3, rp2, 0.0);
-      h4 = field_flux<AI, P1>(dw[3], dg[3], A4, rp4, 0.0);
+      double dw[4][5], dg[4][5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const int pj = p0 + j * ps;
+        const double dmn = dd[ND + pj];
+        project4(fs, dd[pj], dmn, dd[2 * ND + pj], dd[3 * ND + pj], dw[0][j], dw[1][j], dw[2][j],
+                 dw[3][j]);
+        project4(fs, dmn, dd[4 * ND + pj], dd[5 * ND + pj], dd[6 * ND + pj], dg[0][j], dg[1][j],
+                 dg[2][j], dg[3][j]);
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const double A = field_speed(a, al, m, 4);
+        if constexpr (PREC == 1)
+          h[m] = field_flux_f32d<P1>(dw[m], dg[m], A, r32);
+        else
+          h[m] = field_flux<AI, P1>(dw[m], dg[m], A, (m == 0 || m == 3) ? rp4 : rp2, 0.0);
+      }
     }
     double F0, F1, F2, F3;
-    backproject4(fs, h1, h2, h3, h4, F0, F1, F2, F3);
-    // the centre values: 4 F_hat += 2 (F_L + F_R) = 4 F_L + 2 dF of the centre pair
+    backproject4(fs, h[0], h[1], h[2], h[3], F0, F1, F2, F3);
+    // the centre values: 4 F_hat += 2 (F_L + F_R) (= 4 F_L + 2 dF of the centre
+    // pair, where the differences are staged in FP64)
     {
-      const int oL = bo(rL, cL), pc = p0 + 2 * PS;
-      const double mnL = box[(1 + DIR) * PB + oL];
+      const double mnL = bn[oL];
       double FL1, FL2, FL3;
-      normal_flux(box[oL], mnL, box[(2 - DIR) * PB + oL], box[3 * PB + oL],
-                  pl[(1 + DIR) * REG + kL], pl[3 * REG + kL], FL1, FL2, FL3);
-      F0 = fma(4.0, mnL, fma(2.0, dd[ND + pc], F0));
-      F1 = fma(4.0, FL1, fma(2.0, dd[4 * ND + pc], F1));
-      F2 = fma(4.0, FL2, fma(2.0, dd[5 * ND + pc], F2));
-      F3 = fma(4.0, FL3, fma(2.0, dd[6 * ND + pc], F3));
+      normal_flux(box[oL], mnL, bt[oL], box[3 * PB + oL], un[kL], pl[3 * REG + kL], FL1, FL2, FL3);
+      if constexpr (kPacked) {
+        const double mnR = bn[oR];
+        double FR1, FR2, FR3;
+        normal_flux(box[oR], mnR, bt[oR], box[3 * PB + oR], un[kR], pl[3 * REG + kR], FR1, FR2,
+                    FR3);
+        F0 = fma(2.0, mnL + mnR, F0);
+        F1 = fma(2.0, FL1 + FR1, F1);
+        F2 = fma(2.0, FL2 + FR2, F2);
+        F3 = fma(2.0, FL3 + FR3, F3);
+      } else {
+        const int pc = p0 + 2 * ps;
+        F0 = fma(4.0, mnL, fma(2.0, dd[ND + pc], F0));
+        F1 = fma(4.0, FL1, fma(2.0, dd[4 * ND + pc], F1));
+        F2 = fma(4.0, FL2, fma(2.0, dd[5 * ND + pc], F2));
+        F3 = fma(4.0, FL3, fma(2.0, dd[6 * ND + pc], F3));
+      }
     }
-    double *out = DIR ? &fo[(fr * TX + fc) * 4] : &fo[(fr * (TX + 1) + fc) * 4];
+    double *out = fo + (fr * lf + fc) * 4;
     out[0] = F0;
-    out[1 + DIR] = F1;
-    out[2 - DIR] = F2;
+    out[1 + dir] = F1;
+    out[2 - dir] = F2;
     out[3] = F3;
   }
   __syncthreads();
@@ -748,8 +815,8 @@ __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, l
                                               const CUtensorMap *tm) {
   using L = Tile6<TX, TY>;
   constexpr int R = 3, W = L::W, BW = L::BW, XO = L::XO, PB = L::PB, REG = L::REG;
-  double *const sm =
-      reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(sm_in) + 127) & ~uintptr_t(127));
+  // (an offset, so the compiler keeps seeing shared memory)
+  double *const sm = sm_in + (((0u - smem_u32(sm_in)) & 127u) >> 3);
   double *const box = sm + L::kBox;
   double *const pl = sm + L::kPl;
 
@@ -773,6 +840,8 @@ __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, l
     s_id[0] = 0.25 / a.dx;
     s_id[1] = 0.25 / a.dy;
   }
+  __shared__ Speeds s_sp;
+  make_speeds(a, b, 4, s_sp);
 
   const bool use_tma = tm != nullptr && i0 - XO >= 0 && i0 - XO + BW <= a.nx && j0 - R >= 0 &&
                        j0 + TY + R <= a.ny;
@@ -820,8 +889,9 @@ __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, l
   }
   __syncthreads();
 
-  tile6_sweep<TX, TY, AI, P1, PREC, 0>(a, b, i0, j0, gm1, sm, s_rp[0], s_rp[1]);
-  tile6_sweep<TX, TY, AI, P1, PREC, 1>(a, b, i0, j0, gm1, sm, s_rp[0], s_rp[1]);
+#pragma unroll 1
+  for (int dir = 0; dir < 2; ++dir)
+    tile6_sweep<TX, TY, AI, P1, PREC>(a, dir, b, i0, j0, gm1, sm, s_rp[0], s_rp[1], s_sp);
 
   tile2d_update<TX, TY, R>(a, b, i0, j0, dt, sm + L::kFx, sm + L::kFy, s_id[0], s_id[1],
                            [&](int r, int c, int q) { return box[q * PB + (R + r) * BW + XO + c]; });
@@ -940,17 +1010,18 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
   const long long tiles = (a.nx + kT1 - 1) / kT1;
   if constexpr (R == 3) {
     // A problem of fewer tiles than the GPU has SMs is bound by the length
-    // of one thread's chain of FP64 operations: spread each face over
-    // several threads (and the problem over more blocks) instead.
+    // of one thread's chain of operations: spread each face over several
+    // threads (and the problem over more blocks) instead.
     if (tiles * a.nbatch < (long long)sm_count() && (a.nc == 3 || PREC == 0)) {
-      const int tl1 = a.nc == 3 ? kT1Lanes(3) : kT1Lanes(1);
+      constexpr int kL3 = lanes1d(3, P1, PREC);
+      const int tl1 = a.nc == 3 ? cells_lanes1d(kL3) : cells_lanes1d(2);
       dim3 g2((unsigned)((a.nx + tl1 - 1) / tl1), (unsigned)a.nbatch, 1);
       if (a.nc == 3)
         k_line1d_lanes<3, AI, P1, PREC>
-            <<<g2, kThreads1D, smem_line1d<3, kT1Lanes(3), 3, 3>(), s>>>(a);
+            <<<g2, kThreads1D, smem_line1d<3, cells_lanes1d(kL3), 3, kL3>(), s>>>(a);
       else if constexpr (PREC == 0)
         k_line1d_lanes<1, AI, P1, PREC>
-            <<<g2, kThreads1D, smem_line1d<1, kT1Lanes(1), 3, 2>(), s>>>(a);
+            <<<g2, kThreads1D, smem_line1d<1, cells_lanes1d(2), 3, 2>(), s>>>(a);
       return cudaGetLastError();
     }
   }

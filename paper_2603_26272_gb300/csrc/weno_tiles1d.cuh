@@ -13,14 +13,54 @@
 // (dF0 = dm), and the centre values come back as 4 F_i + 2 (F_{i+1} - F_i)
 // after the back-projection.
 // ---------------------------------------------------------------------------
-// The centre values of a sixth-order 1D Euler face between cells L and L+1:
-// 4 F_hat += 2 (F_L + F_{L+1}) = 4 F_L + 2 dF of pair L (R L = I).
-__device__ __forceinline__ void add_centre3(double FL0, double FL1, double FL2, const double *dd,
-                                            int nd, int pair, double &F0, double &F1,
-                                            double &F2) {
-  F0 = fma(4.0, FL0, fma(2.0, dd[nd + pair], F0));
-  F1 = fma(4.0, FL1, fma(2.0, dd[3 * nd + pair], F1));
-  F2 = fma(4.0, FL2, fma(2.0, dd[4 * nd + pair], F2));
+// The centre values of a sixth-order 1D Euler face between cells L and L+1 of
+// the staged fluxes pl[6..8]: 4 F_hat += 2 (F_L + F_{L+1}) (R L = I), as
+// 4 F_L + 2 dF of pair L where the differences dd are staged in FP64.
+template <int REG>
+__device__ __forceinline__ void add_centre3(const double (*pl)[REG], const double *dd, int nd,
+                                            int L, double &F0, double &F1, double &F2) {
+  if (dd) {
+    F0 = fma(4.0, pl[6][L], fma(2.0, dd[nd + L], F0));
+    F1 = fma(4.0, pl[7][L], fma(2.0, dd[3 * nd + L], F1));
+    F2 = fma(4.0, pl[8][L], fma(2.0, dd[4 * nd + L], F2));
+  } else {
+    F0 = fma(2.0, pl[6][L] + pl[6][L + 1], F0);
+    F1 = fma(2.0, pl[7][L] + pl[7][L + 1], F1);
+    F2 = fma(2.0, pl[8][L] + pl[8][L + 1], F2);
+  }
+}
+
+// Field m of face f in FP64 from the staged cells (less its centre values):
+// what the integer path leaves out.
+template <int REG, int AI>
+__device__ __noinline__ double face_wide3(const double (*pl)[REG], int f, int m, double un,
+                                          double ic, double b1, double b2, double A,
+                                          const ReconParams &rp) {
+  FaceState fs = {};
+  fs.un = un;
+  fs.ic = ic;
+  fs.b1 = b1;
+  fs.b2 = b2;
+  double dw[5], dg[5];
+  for (int j = 0; j < 5; ++j) {
+    const int k = f + j;
+    dw[j] = project3_field(fs, m, pl[0][k + 1] - pl[0][k], pl[1][k + 1] - pl[1][k],
+                           pl[2][k + 1] - pl[2][k]);
+    dg[j] = project3_field(fs, m, pl[6][k + 1] - pl[6][k], pl[7][k + 1] - pl[7][k],
+                           pl[8][k + 1] - pl[8][k]);
+  }
+  return pair_wide<AI, true>(-A * dw[2], dw, dg, A, rp);
+}
+
+// Lanes per face of the latency layout and its cells per 128-thread tile: a
+// scalar's positive and negative flux (2); for Euler a characteristic field
+// each (3: p != 1 and FP32 reconstruction), or each flux of a field (6, five
+// faces a warp so that a face's lanes can shuffle).
+__host__ __device__ constexpr int lanes1d(int nc, bool p1, int prec) {
+  return nc == 1 ? 2 : (p1 && prec == 0 ? 6 : 3);
+}
+__host__ __device__ constexpr int cells_lanes1d(int lanes) {
+  return lanes == 2 ? 63 : (lanes == 3 ? 41 : 19);
 }
 
 template <int NC, int T, int R = 3, int LANES = 1>
@@ -32,18 +72,17 @@ constexpr size_t smem_line1d() {
 
 // One tile of T cells (T + 1 faces) of a 1D stage with a stencil of
 // half-width R (order 2R).  LANES threads share a face: 1 (blockDim = T + 1,
-// the throughput layout), or -- for problems too small to fill the GPU, where
-// a stage's time is one thread's chain of FP64 operations -- 3 for Euler (one
-// characteristic field each; blockDim >= 3 (T + 1)) and 2 for a scalar (the
-// positive and the negative flux; blockDim >= 2 (T + 1)).  Every lane layout
-// runs the same arithmetic per field, so the results are bitwise identical.
+// the throughput layout), or, for problems too small to fill the GPU, where a
+// stage's time is one thread's chain of operations, lanes1d() of them.  Every
+// lane layout runs the same arithmetic per field, so the results are bitwise
+// identical.
 // sm: dynamic shared memory of smem_line1d<NC, T, R, LANES>() bytes.
 template <int NC, int AI, bool P1, int PREC, int T, int R = 3, int LANES = 1>
 __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, long long tile,
                                             bool zeroing_block, double *sm) {
   static_assert(R == 3 || PREC == 0, "FP32 reconstruction is sixth order only");
-  static_assert(LANES == 1 || (R == 3 && LANES == (NC == 3 ? 3 : 2) && (NC == 3 || PREC == 0)),
-                "lane layouts: 3 per face for Euler, 2 for a scalar in FP64, sixth order");
+  static_assert(LANES == 1 || (R == 3 && LANES == lanes1d(NC, P1, PREC) && (NC == 3 || PREC == 0)),
+                "lane layouts: sixth order, see lanes1d");
   constexpr int REG = T + 2 * R, N = 2 * R;
   constexpr int NP = (NC == 3) ? 9 : 2;
   double(*pl)[REG] = reinterpret_cast<double(*)[REG]>(sm);
@@ -52,6 +91,9 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
   constexpr bool kDiff = (NC == 3 && R == 3);
   constexpr int ND = REG - 1;  // cell pairs of the tile
   double *const dd = hb + (LANES > 1 ? (T + 1) * NC : 0);  // kDiff: [5][ND]
+  // p = 1 in FP64: packed differences, projected on the integer pipes
+  constexpr bool kPacked = kDiff && P1 && PREC == 0;
+  fx::u64 *const dp = reinterpret_cast<fx::u64 *>(dd);
   const long long i0 = tile * T;
   double dt;
   if (!stage_control(a, b, tile == 0, zeroing_block, dt)) return;
@@ -72,6 +114,8 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     s_r32 = make_r32(a);
     s_idx = (NC == 3 ? 0.25 : 0.5) / a.dx;
   }
+  __shared__ Speeds s_sp;
+  if constexpr (kPacked) make_speeds(a, b, 3, s_sp);
 
   for (int k = tid; k < REG; k += blockDim.x) {
     const long long gi = ghost(i0 - R + k, nx, a.bc_x);
@@ -102,11 +146,16 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
   __syncthreads();
   if constexpr (kDiff) {
     for (int k = tid; k < ND; k += blockDim.x) {
-      dd[k] = pl[0][k + 1] - pl[0][k];
-      dd[ND + k] = pl[1][k + 1] - pl[1][k];
-      dd[2 * ND + k] = pl[2][k + 1] - pl[2][k];
-      dd[3 * ND + k] = pl[7][k + 1] - pl[7][k];
-      dd[4 * ND + k] = pl[8][k + 1] - pl[8][k];
+      const double d[5] = {pl[0][k + 1] - pl[0][k], pl[1][k + 1] - pl[1][k],
+                           pl[2][k + 1] - pl[2][k], pl[7][k + 1] - pl[7][k],
+                           pl[8][k + 1] - pl[8][k]};
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        if constexpr (kPacked)
+          dp[q * ND + k] = fx::pack(d[q]);
+        else
+          dd[q * ND + k] = d[q];
+      }
     }
     __syncthreads();
   }
@@ -122,8 +171,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
                     gm1, fs) && q == 0)
         record_status(a.status, 3, a.stage, b, 0, i0 + f);
       const unsigned long long *al = a.alpha_in + b * 8;
-      double A = bits2d(al[q]);
-      if (a.alpha_single) A = fmax(fmax(bits2d(al[0]), bits2d(al[1])), bits2d(al[2]));
+      const double A = field_speed(a, al, q, 3);
       double h;
       double dW[5], dG[5];  // the field's projected differences over pairs f .. f+4
 #pragma unroll
@@ -142,7 +190,55 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     if (act && q == 0) {
       double F0, F1, F2;
       backproject3(fs, hb[3 * f], hb[3 * f + 1], hb[3 * f + 2], F0, F1, F2);
-      add_centre3(pl[6][f + 2], pl[7][f + 2], pl[8][f + 2], dd, ND, f + 2, F0, F1, F2);
+      add_centre3<REG>(pl, dd, ND, f + 2, F0, F1, F2);
+      fl[f][0] = F0;
+      fl[f][1] = F1;
+      fl[f][2] = F2;
+    }
+  } else if constexpr (LANES == 6) {
+    // lane l < 30 of a warp: face 5 warp + l / 6, field (l % 6) % 3, and of its
+    // pair of lanes the first projects the state and reconstructs the positive
+    // flux, the second the physical flux and the mirrored negative one
+    const int lane = tid & 31, l = min(lane, 29), r = l % 6, q = r % 3, sgn = r / 3;
+    const int f = min(5 * (tid >> 5) + l / 6, T);
+    const bool act = lane < 30 && i0 + f - 1 < nx;
+    const int other = lane < 30 ? lane + (sgn ? -3 : 3) : lane;
+    FaceState fs = {};
+    const int kL = f + 2, kR = f + 3;
+    if (!roe_face(pl[5][kL], pl[3][kL], 0.0, pl[4][kL], pl[5][kR], pl[3][kR], 0.0, pl[4][kR], gm1,
+                  fs) && act && r == 0)
+      record_status(a.status, 3, a.stage, b, 0, i0 + f);
+    auto du = [&](int c, int j) { return dp[c * ND + f + j]; };
+    auto df = [&](int c, int j) { return dp[(c == 0 ? 1 : 2 + c) * ND + f + j]; };
+    int E[3];
+    const int ea = s_sp.ea[0];
+    bool ok = face_exponents<3>(ea, du, df, E);
+    const fx::LeftRows<3> rows =
+        fx::left_rows<3>(E, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic), __dmul_rn(fs.b1, fs.un),
+                         __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
+    ok = ok && rows.emax < 2047;
+    fx::i64 v[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      const fx::u64 in[3] = {sgn ? dp[ND + f + j] : dp[f + j],
+                             sgn ? dp[3 * ND + f + j] : dp[ND + f + j],
+                             sgn ? dp[4 * ND + f + j] : dp[2 * ND + f + j]};
+      const fx::Proj p = fx::project<3>(rows, E, sgn ? ea : 0, in);
+      v[j] = q == 1 ? p.r - p.z : (q == 0 ? p.z + p.tc : p.z - p.tc);
+    }
+    bool wide;
+    const ReconParams &rp = s_rp[q == 1 ? 0 : 1];
+    double h = field_lanes<AI>(v, s_sp.ka[0][q], rows.um + ea - 1592, ok, sgn, other, rp,
+                                         wide);
+    if (wide && act && sgn == 0)
+      h = face_wide3<REG, AI>(pl, f, q, fs.un, fs.ic, fs.b1, fs.b2,
+                                        field_speed(a, a.alpha_in + b * 8, q, 3), rp);
+    const double h1 = __shfl_sync(0xffffffffu, h, min(lane + 1, 31)),
+                 h2 = __shfl_sync(0xffffffffu, h, min(lane + 2, 31));
+    if (act && r == 0) {
+      double F0, F1, F2;
+      backproject3(fs, h, h1, h2, F0, F1, F2);
+      add_centre3<REG>(pl, nullptr, 0, kL, F0, F1, F2);
       fl[f][0] = F0;
       fl[f][1] = F1;
       fl[f][2] = F2;
@@ -180,10 +276,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
         else
           d[j] = x + g;
       }
-      if constexpr (AI == kAiTiny)
-        c = fx::recon6<false>(d[0], d[1], d[2], d[3], d[4], rp.e3);
-      else
-        c = fx::recon6<true>(d[0], d[1], d[2], d[3], d[4], sens_fixed<AI>(d, es, rp));
+      c = recon_fixed<AI>(d, es - 1079, rp);
     }
     c += __shfl_xor_sync(0xffffffffu, c, 1);
     if (act && sgn == 0) {
@@ -233,10 +326,25 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
                       gm1, fs))
           record_status(a.status, 3, a.stage, b, 0, i0 + f);
         const unsigned long long *al = a.alpha_in + b * 8;
-        double A1 = bits2d(al[0]), A2 = bits2d(al[1]), A3 = bits2d(al[2]);
-        if (a.alpha_single) A1 = A2 = A3 = fmax(fmax(A1, A2), A3);
+        const double A1 = field_speed(a, al, 0, 3), A2 = field_speed(a, al, 1, 3),
+                     A3 = field_speed(a, al, 2, 3);
         double h1, h2, h3;
-        if constexpr (R == 3) {
+        if constexpr (kPacked) {
+          double hs[3];
+          face_fields<3, AI>(
+              fs, s_sp.ka[0], s_sp.ea[0], [&](int c, int j) { return dp[c * ND + f + j]; },
+              [&](int c, int j) { return dp[(c == 0 ? 1 : 2 + c) * ND + f + j]; },
+              [&](int m) -> const ReconParams & { return s_rp[m == 1 ? 0 : 1]; },
+              [&](int m) {
+                return face_wide3<REG, AI>(pl, f, m, fs.un, fs.ic, fs.b1, fs.b2,
+                                                     field_speed(a, al, m, 3),
+                                                     s_rp[m == 1 ? 0 : 1]);
+              },
+              hs);
+          h1 = hs[0];
+          h2 = hs[1];
+          h3 = hs[2];
+        } else if constexpr (R == 3) {
           double dW[3][5], dG[3][5];  // projected differences over pairs f .. f+4
 #pragma unroll
           for (int j = 0; j < 5; ++j) {
@@ -276,7 +384,8 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
         }
         double F0, F1, F2;
         backproject3(fs, h1, h2, h3, F0, F1, F2);
-        if constexpr (R == 3) add_centre3(pl[6][kL], pl[7][kL], pl[8][kL], dd, ND, kL, F0, F1, F2);
+        if constexpr (R == 3)
+          add_centre3<REG>(pl, kPacked ? nullptr : dd, ND, kL, F0, F1, F2);
         fl[f][0] = F0;
         fl[f][1] = F1;
         fl[f][2] = F2;
@@ -335,13 +444,11 @@ __global__ void __launch_bounds__(kThreads1D) k_line1d(const StageArgs a) {
                                         blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, sm);
 }
 
-// Latency layout of small 1D problems: 128 threads, 3 per face for Euler
-// (41 cells a tile) or 2 per face for a scalar (63 cells).
-__host__ __device__ constexpr int kT1Lanes(int nc) { return nc == 3 ? 41 : 63; }
-
+// Latency layout of small 1D problems (lanes1d).
 template <int NC, int AI, bool P1, int PREC>
 __global__ void __launch_bounds__(kThreads1D) k_line1d_lanes(const StageArgs a) {
   extern __shared__ double sm[];
-  line1d_tile<NC, AI, P1, PREC, kT1Lanes(NC), 3, (NC == 3 ? 3 : 2)>(
+  constexpr int kL = lanes1d(NC, P1, PREC);
+  line1d_tile<NC, AI, P1, PREC, cells_lanes1d(kL), 3, kL>(
       a, blockIdx.y, blockIdx.x, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, sm);
 }

@@ -136,3 +136,143 @@ def test_reconstruction_against_quadruple_precision(harness, kind, mode, eps4):
                          capture_output=True, text=True).stdout.split()
     assert float(out[0]) <= 2.0 ** -50
     assert float(out[1]) <= 2.0 ** -60
+
+FACE = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <random>
+#include <cmath>
+#include "weno_fixed.cuh"
+#ifdef __x86_64__
+typedef __float128 Q;
+#else
+typedef long double Q;
+#endif
+using namespace weno::fx;
+static Q qabs(Q x) { return x < 0 ? -x : x; }
+static Q paper(const Q *d) {  // f - v2, eq. (11)-(22), p = 1, the sensitivity term left out
+  Q s[4], t[4] = {3 * d[1] - d[0], d[1] + d[2], 3 * d[2] - d[3], 3 * d[4] - 5 * d[3]}, b[4];
+  for (int k = 0; k < 4; ++k) s[k] = d[k + 1] - d[k];
+  for (int k = 0; k < 4; ++k) b[k] = (Q)13 / 3 * s[k] * s[k] + t[k] * t[k];
+  b[3] = (b[0] + b[1] + b[2] + b[3]) / 4;
+  const Q r5 = s[3] - s[0] + 3 * (s[1] - s[2]), T = 4 * r5 * r5, D[4] = {1, 9, 9, 1};
+  const Q r[4] = {5 * d[1] - 2 * d[0], d[1] + 2 * d[2], 4 * d[2] - d[3], 6 * d[2] - 5 * d[3] + 2 * d[4]};
+  Q num = 0, den = 0;
+  for (int k = 0; k < 4; ++k) { const Q a = D[k] * (1 + T / (b[k] + (Q)1e-80)); num += a * r[k]; den += a; }
+  return num / den / 6;
+}
+int main(int argc, char **argv) {
+  const int jump = atoi(argv[1]);
+  const double phase = atof(argv[2]), cold = atof(argv[3]);
+  std::mt19937_64 g(3);
+  std::uniform_real_distribution<double> U(-1, 1);
+  double worst = 0;
+  long smooths = 0, fields = 0;
+  for (int it = 0; it < 4000; ++it) {
+    const double gm1 = 0.4, un = U(g), ut = U(g), c = cold * (1 + 0.5 * U(g)), ic = 1 / c;
+    const double b1 = gm1 * ic * ic, b2 = b1 * 0.5 * (un * un + ut * ut);
+    const double A[4] = {1.2 * (std::fabs(un) + c), std::fabs(un) + 0.1, std::fabs(un) + 0.1, 1.2 * (std::fabs(un) + c)};
+    const double ph = 3 * U(g), a1 = 0.2 * U(g), a2 = 0.2 * U(g), jr = 0.5 * U(g), jp = 0.5 * U(g);
+    double V[4][6], F[4][6];
+    for (int j = 0; j < 6; ++j) {
+      const double s1 = a1 * std::sin(ph + phase * j), s2 = a2 * std::cos(2 * ph + 0.7 * phase * j);
+      const bool on = jump && j > it % 5;
+      const double rho = 1 + s1 + (on ? jr : 0), u = un + c * s2, v = ut + c * s1;
+      const double p = c * c / 1.4 * (1 + s2 + (on ? jp : 0)), E = p / gm1 + 0.5 * rho * (u * u + v * v);
+      V[0][j] = rho; V[1][j] = rho * u; V[2][j] = rho * v; V[3][j] = E;
+      F[0][j] = V[1][j]; F[1][j] = V[1][j] * u + p; F[2][j] = V[2][j] * u; F[3][j] = (E + p) * u;
+    }
+    const int a = exponent(std::fmax(A[0], A[1])) - 1022;
+    double dU[4][5], dF[4][5];
+    u64 pU[4][5], pF[4][5];
+    int E[4];
+    for (int q = 0; q < 4; ++q) {
+      int eu = 0, ef = 0;
+      for (int j = 0; j < 5; ++j) {
+        pU[q][j] = pack(dU[q][j] = V[q][j + 1] - V[q][j]);
+        pF[q][j] = pack(dF[q][j] = F[q][j + 1] - F[q][j]);
+        eu = imax(eu, packed_exponent(pU[q][j]));
+        ef = imax(ef, packed_exponent(pF[q][j]));
+      }
+      E[q] = imax(eu, ef - a);
+    }
+    const double t1 = un * ic, t2 = b1 * un, t3 = b1 * ut;
+    const LeftRows<4> rows = left_rows<4>(E, b2, b1, t1, t2, t3, ic, ut);
+    Proj PU[5], PF[5];
+    for (int j = 0; j < 5; ++j) {
+      u64 v[4];
+      for (int q = 0; q < 4; ++q) v[q] = pU[q][j];
+      PU[j] = project<4>(rows, E, 0, v);
+      for (int q = 0; q < 4; ++q) v[q] = pF[q][j];
+      PF[j] = project<4>(rows, E, a, v);
+    }
+    double h[4], top = 0;
+    Q ref[4];
+    for (int m = 0; m < 4; ++m) {
+      auto part = [&](const Proj &p) { return m == 0 ? p.z + p.tc : m == 1 ? p.r - p.z : m == 2 ? p.s : p.z - p.tc; };
+      i64 x[5], y[5];
+      for (int j = 0; j < 5; ++j) x[j] = times_speed(speed(A[m], a), part(PU[j])), y[j] = part(PF[j]);
+      const int n = field_shift(x, y), k = (m == 2 ? rows.us : rows.um) + a - 1592 + 6 - n;
+      h[m] = 0;
+      if (n < 64) {
+        shift_field(x, n);
+        shift_field(y, n);
+        i64 d[5], e[5];
+        for (int j = 0; j < 5; ++j) d[j] = x[j] + y[j], e[4 - j] = x[j] - y[j];
+        int cp, cm;
+        const bool sp = smooth_term<false>(d, cp), sm = smooth_term<false>(e, cm);
+        ++fields;
+        smooths += sp && sm;
+        const i64 S = sp && sm ? smooth_sum(y, cp + cm) : rough_sum(x, y, [](const i64(&d)[5]) {
+          return recon6<false>(d[0], d[1], d[2], d[3], d[4], Flt()); });
+        h[m] = (double)S * sixth(k);
+      }
+      Q row[4] = {0, 0, 0, 0}, P[5], N[5], X2 = 0;
+      if (m == 0 || m == 3) { const Q s = m ? -1 : 1; row[0] = b2 + s * t1; row[1] = -t2 - s * ic; row[2] = -(Q)t3; row[3] = b1; }
+      if (m == 1) { row[0] = 1 - (Q)b2; row[1] = t2; row[2] = t3; row[3] = -b1; }
+      if (m == 2) { row[0] = -ut; row[2] = 1; }
+      for (int j = 0; j < 5; ++j) {
+        Q w = 0, f = 0;
+        for (int q = 0; q < 4; ++q) {
+          w += row[q] * dU[q][j];
+          f += row[q] * dF[q][j];
+          top = std::fmax(top, (double)qabs(A[m] * row[q] * dU[q][j]));
+        }
+        if (j == 2) X2 = A[m] * w;
+        P[j] = A[m] * w + f;
+        N[4 - j] = A[m] * w - f;
+      }
+      ref[m] = -X2 + paper(P) + paper(N);
+    }
+    for (int m = 0; m < 4; ++m) worst = std::fmax(worst, (double)(qabs((Q)h[m] - ref[m]) / top));
+  }
+  printf("%.17g %.17g\n", worst, (double)smooths / fields);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def face_harness(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("no host compiler")
+    d = tmp_path_factory.mktemp("face")
+    (d / "f.cpp").write_text(FACE)
+    subprocess.run([cxx, "-O2", "-std=c++17", "-ffp-contract=off", "-w", "-I",
+                    os.path.join(ROOT, "paper_2603_26272_gb300", "csrc"), str(d / "f.cpp"), "-o",
+                    str(d / "f")], check=True)
+    return str(d / "f")
+
+
+@pytest.mark.parametrize("cold", [1.0, 1e-3])
+@pytest.mark.parametrize("jump,phase", [(0, 0.01), (0, 0.08), (0, 0.3), (0, 1.5), (1, 0.01), (1, 0.3)])
+def test_projected_face_against_quadruple_precision(face_harness, jump, phase, cold):
+    """The four fields of Euler faces from packed differences: projection,
+    smooth test and weights together, at phases per cell where all, some and
+    none of the fields pass the smooth test.  Tolerance: that of the
+    reconstruction, 2^-50, relative to the largest alpha L dU term of the face."""
+    out = subprocess.run([face_harness, str(jump), repr(phase), repr(cold)], check=True,
+                         capture_output=True, text=True).stdout.split()
+    assert float(out[0]) <= 2.0 ** -50
+    assert (float(out[1]) > 0.5) == (phase == 0.01 and not jump)

@@ -23,25 +23,6 @@
 
 namespace weno {
 
-// Parameters of eqs. (21)-(22) for one characteristic field.  The field's
-// split fluxes reach the reconstruction multiplied by `scale` (2 or 4, see
-// the projection below), so mu_0 and, without Ai, epsilon are scaled to keep
-// Gamma_k exactly the paper's.
-struct ReconParams {
-  double eps4;   // 4 * eps            (indicators are carried as 4*beta, 4*tau)
-  double mu0s;   // scale * mu_0       (Ai)
-  double efix;   // 4 * eps * scale^2  (no Ai: mu = 1)
-  double p;      // power parameter of eq. (21)
-  double me;     // sqrt(4 eps) / 6    (Ai: 4 eps mu^2 = (me * dev + mo)^2, dev =
-  double mo;     // sqrt(4 eps) * scale * mu_0   the sum of |v_j - mean v|)
-  double e0;     // mo^2: the term of a flat stencil (dev = 0)
-  float mef;     // me^2 = eps / 9 = mef 2^eme, mef in [1, 2) (FP32)
-  int eme;
-  int lthr;      // dev >= 2^(lthr - 1019) implies me dev >= 2^30 mo (mo negligible)
-  int es_lo, es_hi;  // exponents of a field's largest difference the integer path takes
-  fx::Flt e3;        // 3 efix (no Ai), in the data's units squared
-};
-
 // ---------------------------------------------------------------------------
 // Format changes on the integer pipe.  An FP64 <-> FP32 conversion issues to
 // the FP64 pipe, the one these kernels are bound by; where a value only needs
@@ -789,10 +770,6 @@ __device__ __forceinline__ double pair_flux_r(const RPart &p, const RPart &m) {
 // Weights are normalised before the products with the candidates, so no
 // intermediate can overflow.
 // ---------------------------------------------------------------------------
-struct Recon32 {
-  float eps4;   // 4 * eps32
-  float p;      // power parameter
-};
 
 template <bool P1>
 __device__ __forceinline__ float za6_f32(float e0, float e1, float e2, float e3, float e4,
@@ -1033,17 +1010,18 @@ __device__ __forceinline__ void backproject3(const FaceState &f, double h1, doub
 }
 
 // Exponent codes of a face's five pairs (weno_fixed.cuh) with fluxes aligned
-// to 2^a times the states: false if a difference is outside the packed range.
-template <int NC, class DU, class DF>
-__device__ __forceinline__ bool face_exponents(int a, DU du, DF df, int (&E)[NC]) {
-  int top = 0;
+// to 2^a times the states, top the largest of the codes: false if a difference
+// is outside the packed range.
+template <int NC, class Diff>
+__device__ __forceinline__ bool face_exponents(int a, Diff diff, int (&E)[NC], int &top) {
+  top = 0;
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
     int eu = 0, ef = 0;
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-      eu = max(eu, fx::packed_exponent(du(q, j)));
-      ef = max(ef, fx::packed_exponent(df(q, j)));
+      eu = max(eu, fx::packed_exponent(diff(0, q, j)));
+      ef = max(ef, fx::packed_exponent(diff(1, q, j)));
     }
     top = max(top, max(eu, ef));
     E[q] = max(eu, ef - a);
@@ -1060,57 +1038,61 @@ struct FieldSum {
   fx::i64 S;
   int k;
 };
-template <int AI>
-__device__ __noinline__ fx::i64 rough_call(fx::i64 x0, fx::i64 x1, fx::i64 x2, fx::i64 x3,
-                                           fx::i64 x4, fx::i64 g0, fx::i64 g1, fx::i64 g2,
-                                           fx::i64 g3, fx::i64 g4, int k, const ReconParams &P) {
-  fx::i64 x[5] = {x0, x1, x2, x3, x4}, g[5] = {g0, g1, g2, g3, g4};
-  return fx::rough_sum(x, g, [&](const fx::i64(&d)[5]) { return recon_fixed<AI>(d, k, P); });
-}
-__device__ __forceinline__ bool in_range(int k, const ReconParams &P) {
-  const int es = k + 1080;
+// Whether the integer path takes differences of up to about 2^e.
+__device__ __forceinline__ bool in_range(int e, const ReconParams &P) {
+  const int es = e + 1023;
   return es >= P.es_lo && es <= P.es_hi;
 }
 template <int AI>
-__device__ __noinline__ FieldSum field_call(fx::i64 w0, fx::i64 w1, fx::i64 w2, fx::i64 w3,
-                                            fx::i64 w4, fx::i64 g0, fx::i64 g1, fx::i64 g2,
-                                            fx::i64 g3, fx::i64 g4, fx::Limb A, int k0,
-                                            const ReconParams &P) {
+__device__ __noinline__ FieldSum rough_call(fx::i64 x0, fx::i64 x1, fx::i64 x2, fx::i64 x3,
+                                            fx::i64 x4, fx::i64 g0, fx::i64 g1, fx::i64 g2,
+                                            fx::i64 g3, fx::i64 g4, int k0, const ReconParams &P) {
+  fx::i64 x[5] = {x0, x1, x2, x3, x4}, g[5] = {g0, g1, g2, g3, g4};
+  const int n = fx::field_shift(x, g), k = k0 + 6 - n;
+  if (n == 64) return FieldSum{0, 0};
+  if (!in_range(k + 57, P)) return FieldSum{0, INT_MIN};
+  fx::shift_field(x, n);
+  fx::shift_field(g, n);
+  return FieldSum{fx::rough_sum(x, g, [&](const fx::i64(&d)[5]) { return recon_fixed<AI>(d, k, P); }),
+                  k};
+}
+// 6 h of one field less its centre values; wide: the field is left to FP64.
+struct FieldValue {
+  double h6;
+  bool wide;
+};
+template <int AI>
+__device__ __noinline__ FieldValue field_call(fx::i64 w0, fx::i64 w1, fx::i64 w2, fx::i64 w3,
+                                              fx::i64 w4, fx::i64 g0, fx::i64 g1, fx::i64 g2,
+                                              fx::i64 g3, fx::i64 g4, fx::Limb A, int k0,
+                                              const ReconParams &P) {
   fx::i64 x[5] = {w0, w1, w2, w3, w4}, g[5] = {g0, g1, g2, g3, g4};
 #pragma unroll
   for (int j = 0; j < 5; ++j) x[j] = fx::times_speed(A, x[j]);
-  const int n = fx::field_shift(x, g);
-  if (n == 64) return FieldSum{0, 0};
-  const int k = k0 + 6 - n;
-  if (!in_range(k, P)) return FieldSum{0, INT_MIN};
-  fx::shift_field(x, n);
-  fx::shift_field(g, n);
-  int cp = 0, cm = 0;
-  bool smooth = true;
+  if (!in_range(k0 + 61, P)) {
+    fx::i64 any = 0;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) any |= x[j] | g[j];
+    return FieldValue{0.0, any != 0};
+  }
+  int corr = 0;
+  bool smooth = true;  // (both signs run: lanes that left the loop apart would call apart)
 #pragma unroll 1
   for (int s = 0; s < 2; ++s) {
     fx::i64 d[5];
+    int c;
 #pragma unroll
-    for (int j = 0; j < 5; ++j) d[j] = x[j] + g[j];
-    smooth = fx::smooth_term<(AI != kAiTiny)>(d, cm) && smooth;
-    cp += cm;
+    for (int j = 0; j < 5; ++j) d[j] = (x[j] + g[j]) >> 2;
+    smooth = fx::smooth_term<(AI != kAiTiny)>(d, c) && smooth;
+    corr += c;
     fx::mirror(x, g);
   }
-  return FieldSum{smooth ? fx::smooth_sum(g, cp)
-                         : rough_call<AI>(x[0], x[1], x[2], x[3], x[4], g[0], g[1], g[2], g[3],
-                                          g[4], k, P),
-                  k};
-}
-// h of one field less its centre values; wide() gives it in FP64 where ok is
-// false or field_call leaves it.
-template <int AI, class Wide>
-__device__ __forceinline__ double field_fixed(const fx::i64 (&w)[5], const fx::i64 (&g)[5],
-                                              const fx::Limb &A, int k0, bool ok,
-                                              const ReconParams &P, Wide wide) {
-  const FieldSum s = field_call<AI>(w[0], w[1], w[2], w[3], w[4], g[0], g[1], g[2], g[3], g[4],
-                                    A, k0, P);
-  if (!ok || s.k == INT_MIN) return wide();
-  return (double)s.S * fx::sixth(s.k);
+  FieldSum r = {0, k0 + 2};
+  if (smooth)
+    r.S = fx::smooth_sum(g, corr);
+  else
+    r = rough_call<AI>(x[0], x[1], x[2], x[3], x[4], g[0], g[1], g[2], g[3], g[4], k0, P);
+  return FieldValue{fx::from_fixed(r.S, r.k), r.k == INT_MIN};
 }
 
 __device__ __forceinline__ fx::i64 shfl64(fx::i64 v, int src) {
@@ -1119,8 +1101,8 @@ __device__ __forceinline__ fx::i64 shfl64(fx::i64 v, int src) {
 // The same spread over two lanes of a warp (every lane of the warp calls this):
 // lane sgn = 0 brings the projected state differences, lane sgn = 1 those of
 // the flux, `other` is the partner; each reconstructs one of the fluxes.  The
-// operations are field_call's.  Returns h on both lanes, wide = true where
-// the field is left to FP64.
+// operations are field_call's.  Returns 6 h on both lanes, wide = true
+// where the field is left to FP64.
 template <int AI>
 __device__ __forceinline__ double field_lanes(const fx::i64 (&v)[5], const fx::Limb &A, int k0,
                                               bool ok, int sgn, int other, const ReconParams &P,
@@ -1132,63 +1114,102 @@ __device__ __forceinline__ double field_lanes(const fx::i64 (&v)[5], const fx::L
     x[j] = sgn ? got : own;
     g[j] = sgn ? own : got;
   }
-  const int n = fx::field_shift(x, g), k = n == 64 ? 0 : k0 + 6 - n;
-  wide = !ok || (n < 64 && !in_range(k, P));
-  fx::shift_field(x, n == 64 ? 1 : n);
-  fx::shift_field(g, n == 64 ? 1 : n);
+  fx::i64 any = 0;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) any |= x[j] | g[j];
+  wide = !ok || (any != 0 && !in_range(k0 + 61, P));
   if (sgn) fx::mirror(x, g);
   fx::i64 d[5];
 #pragma unroll
-  for (int j = 0; j < 5; ++j) d[j] = x[j] + g[j];
+  for (int j = 0; j < 5; ++j) d[j] = (x[j] + g[j]) >> 2;
   int c;
   const bool own = fx::smooth_term<(AI != kAiTiny)>(d, c);
   const int c2 = __shfl_sync(0xffffffffu, own ? c : INT_MIN, other);
   const bool smooth = own && c2 != INT_MIN;
   fx::i64 r = 0;
-  if (!smooth && !wide && n < 64) r = recon_fixed<AI>(d, k, P) - 3 * d[2];
-  r += shfl64(r, other);
+  int k = k0 + 2;
   if (sgn) fx::mirror(x, g);
+  if (!smooth && !wide) {
+    const int n = fx::field_shift(x, g);
+    k = k0 + 6 - n;
+    wide = n < 64 && !in_range(k + 57, P);
+    if (n < 64 && !wide) {
+      fx::i64 y[5], f[5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        y[j] = x[j];
+        f[j] = g[j];
+      }
+      fx::shift_field(y, n);  // before the mirroring, as rough_call does
+      fx::shift_field(f, n);
+      if (sgn) fx::mirror(y, f);
+#pragma unroll
+      for (int j = 0; j < 5; ++j) d[j] = y[j] + f[j];
+      r = recon_fixed<AI>(d, k, P) - 3 * d[2];
+    }
+  }
+  r += shfl64(r, other);
   const fx::i64 S = smooth ? fx::smooth_sum(g, c + c2) : r;
-  return n == 64 ? 0.0 : (double)S * fx::sixth(k);
+  return any == 0 ? 0.0 : fx::from_fixed(S, k);
 }
 
-// The fields of one face from its packed differences du(q, j), df(q, j) of
-// states and physical fluxes, component q, pair j; KA[m] and a: the fields'
+// 6 h of the fields of one face from its packed differences diff(s, q, j) of the
+// state (s = 0) and the physical flux (s = 1), component q, pair j; KA[m] and a: the fields'
 // speeds (fx::speed).
-template <int NC, int AI, class DU, class DF, class Wide, class RP>
-__device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb *KA, int a, DU du,
-                                            DF df, RP rp, Wide wide, double (&h)[NC]) {
-  int E[NC];
-  bool ok = face_exponents<NC>(a, du, df, E);
+template <int NC, int AI, class Diff, class Wide, class RP>
+__device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb *KA, int a,
+                                            Diff diff, RP rp, Wide wide, double (&h)[NC]) {
+  int E[NC], top;
+  bool ok = face_exponents<NC>(a, diff, E, top);
+  if (top == 0) {  // nothing varies over the stencil
+#pragma unroll
+    for (int m = 0; m < NC; ++m) h[m] = 0.0;
+    return;
+  }
   const fx::LeftRows<NC> rows =
       fx::left_rows<NC>(E, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic), __dmul_rn(fs.b1, fs.un),
                         __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
   ok = ok && rows.emax < 2047;
-  fx::Proj U[5], F[5];
-#pragma unroll
-  for (int j = 0; j < 5; ++j) {
-    fx::u64 v[NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) v[q] = du(q, j);
-    U[j] = fx::project<NC>(rows, E, 0, v);
-#pragma unroll
-    for (int q = 0; q < NC; ++q) v[q] = df(q, j);
-    F[j] = fx::project<NC>(rows, E, a, v);
-  }
-  const int k0 = rows.um + a - 1592;
-  auto field = [&](int m, int k, auto part) {
-    fx::i64 w[5], g[5];
+  fx::i64 w[5], g[5];
+  auto field = [&](int m, int k) {
+    const FieldValue f = field_call<AI>(w[0], w[1], w[2], w[3], w[4], g[0], g[1], g[2], g[3], g[4],
+                                        KA[m], k + a - 1592, rp(m));
+    h[m] = ok && !f.wide ? f.h6 : 6.0 * wide(m);
+  };
+  if constexpr (NC == 4) {
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-      w[j] = part(U[j]);
-      g[j] = part(F[j]);
+      w[j] = fx::project_shear(rows, E, 0, diff(0, 0, j), diff(0, 2, j));
+      g[j] = fx::project_shear(rows, E, a, diff(1, 0, j), diff(1, 2, j));
     }
-    h[m] = field_fixed<AI>(w, g, KA[m], k, ok, rp(m), [&]() { return wide(m); });
+    field(2, rows.us);
+  }
+  // the states, then the physical fluxes (a loop: half the code to fetch)
+  fx::Proj U[5], F[5] = {};
+#pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      U[j] = F[j];
+      fx::u64 v[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) v[q] = diff(s, q, j);
+      F[j] = fx::project<NC>(rows, E, s ? a : 0, v);
+    }
+  }
+  auto part = [&](auto of) {
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      w[j] = of(U[j]);
+      g[j] = of(F[j]);
+    }
   };
-  if constexpr (NC == 4) field(2, rows.us + a - 1592, [](const fx::Proj &p) { return p.s; });
-  field(1, k0, [](const fx::Proj &p) { return p.r - p.z; });
-  field(0, k0, [](const fx::Proj &p) { return p.z + p.tc; });
-  field(NC - 1, k0, [](const fx::Proj &p) { return p.z - p.tc; });
+  part([](const fx::Proj &p) { return p.r - p.z; });
+  field(1, rows.um);
+  part([](const fx::Proj &p) { return p.z + p.tc; });
+  field(0, rows.um);
+  part([](const fx::Proj &p) { return p.z - p.tc; });
+  field(NC - 1, rows.um);
 }
 
 }  // namespace weno

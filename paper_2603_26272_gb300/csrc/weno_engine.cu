@@ -350,6 +350,7 @@ weno_status weno_engine_admit(weno_engine *E, const weno_desc *d, const double *
   S.eps = d->eps;
   S.mu0 = d->mu0;
   S.p = d->p;
+  S.sp = weno::scheme_params(S.eps, S.mu0, S.p, true, S.dx, S.dy);
   S.t_final = t_final;
   S.U = (double *)(E->arena + off);
   S.U1 = (double *)(E->arena + off + sb);

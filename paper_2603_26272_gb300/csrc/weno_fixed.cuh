@@ -59,7 +59,11 @@ WENO_FX uint32_t rcp_seed(uint32_t fbits) {  // bits of about 1 / f, f in [1, 2)
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(fbits)));
   return __float_as_uint(r);
 }
-WENO_FX u64 dbits(double x) { return (u64)__double_as_longlong(x); }
+// (by halves: a test of the exponent bits of a bit-cast double is turned into
+// an FP64 comparison)
+WENO_FX u64 dbits(double x) {
+  return ((u64)(uint32_t)__double2hiint(x) << 32) | (uint32_t)__double2loint(x);
+}
 WENO_FX double bitsd(u64 b) { return __longlong_as_double((i64)b); }
 #else
 WENO_FX u64 shr(u64 x, int n) { return n >= 64 ? 0 : x >> n; }
@@ -152,20 +156,20 @@ struct Flt {
   u64 m;
   int e;
 };
-// raw 2^e, raw = 0 or above 2^57; a zero becomes 2^(63 + e0).
-WENO_FX Flt normal(u64 raw, int e, int e0) {
+// raw 2^e, raw = 0 or above 2^56; a zero counts as 2^56.
+WENO_FX Flt normal(u64 raw, int e) {
   Flt f;
-  const int n = clz32(hi32(raw));
-  const bool z = raw == 0;
-  f.m = z ? 0x8000000000000000ull : shl(raw, n);
-  f.e = z ? e0 : e - n;
+  const uint32_t h = hi32(raw) > 0x01000000u ? hi32(raw) : 0x01000000u;
+  const int n = clz32(h);
+  f.m = shl(((u64)h << 32) | lo32(raw), n);
+  f.e = e - n;
   return f;
 }
 // raw 2^e + s, aligned to the larger of the two.
 WENO_FX Flt normal_plus(u64 raw, int e, const Flt &s) {
   const int d = raw ? s.e - e : 8192;
   const u64 v = shr(raw, d > 0 ? d + 1 : 1) + shr(s.m, d > 0 ? 1 : 1 - d);
-  return normal(v, (d > 0 ? s.e : e) + 1, 0);
+  return normal(v, (d > 0 ? s.e : e) + 1);
 }
 
 // Six times the correction f - v2 of eqs. (14)-(22) (p = 1) of the stencil
@@ -176,7 +180,7 @@ WENO_FX Flt normal_plus(u64 raw, int e, const Flt &s) {
 // to the b_k.  At epsilon <= 2^-126 it is below a quarter of the unit squared
 // wherever mu_0 is below the largest difference, and it could only decide
 // between candidates that agree to a few units; it is then left out, and an
-// indicator that is 0 in these units counts as 2^-10.
+// indicator that is 0 in these units counts as 2^-4.
 template <bool SENS>
 WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e) {
   const i64 s0 = d1 - d0, s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3;
@@ -198,16 +202,16 @@ WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e) {
     b2 = normal_plus(i2.raw, 64 - 2 * i2.n, e);
     b3 = normal_plus(raw3, 64 - 2 * nm, e);
   } else {
-    b0 = normal(i0.raw, 64 - 2 * i0.n, -73);
-    b1 = normal(i1.raw, 64 - 2 * i1.n, -73);
-    b2 = normal(i2.raw, 64 - 2 * i2.n, -73);
-    b3 = normal(raw3, 64 - 2 * nm, -73);
+    b0 = normal(i0.raw, 64 - 2 * i0.n);
+    b1 = normal(i1.raw, 64 - 2 * i1.n);
+    b2 = normal(i2.raw, 64 - 2 * i2.n);
+    b3 = normal(raw3, 64 - 2 * nm);
   }
   // T = 12 r5^2
   const u64 ra = abs64(r5);
   const int nt = clz64(ra) - 1;
   const u64 sq = sqrhi(shl(ra, nt));
-  const Flt T = normal(3ull * sq, 66 - 2 * nt, -16384);  // 0: far below every b_k
+  const Flt T = normal(3ull * sq, ra ? 66 - 2 * nt : -16384);  // 0: far below every b_k
   // y_k = D_k z_k with the largest of D_k / b_k and 8 / T in [2^60, 2^61)
   const int e0 = b0.e < b3.e ? b0.e : b3.e, e1 = (b1.e < b2.e ? b1.e : b2.e) - 3;
   const int e01 = e0 < e1 ? e0 : e1, em = (e01 < T.e - 3 ? e01 : T.e - 3) - 3;
@@ -223,7 +227,7 @@ WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e) {
   const u64 B = 0x8000000000000000ull;
   const u64 N = mulhi64(y0, B + 2 * (u64)p0) + mulhi64(y2, B + 2 * (u64)q) +
                 mulhi64(y3, B + 2 * (u64)p3);
-  const i64 Ns = (i64)(N - (y0 >> 1) - (y2 >> 1) - (y3 >> 1));
+  const i64 Ns = (i64)(N - ((y0 + y2 + y3) >> 1));
   const u64 c = mulhi64(abs64(Ns), rcp64(shl(den, nd)));
   return (d1 + 2 * d2) + (Ns < 0 ? -(i64)c : (i64)c);
 }
@@ -297,7 +301,7 @@ WENO_FX Limb limb(i64 v) {
 struct Acc {
   i64 hi, cr;
 };
-WENO_FX i64 acc_value(const Acc &a) { return (a.hi << 1) + (a.cr >> 30); }  // sum / 2^63
+WENO_FX i64 over63(const Acc &a) { return (a.hi << 1) + (a.cr >> 30); }  // sum / 2^63
 WENO_FX void mac(Acc &s, const Limb &a, const Limb &b) {
   s.hi += (i64)a.h * b.h;
   s.cr += (i64)a.h * b.l;
@@ -325,14 +329,14 @@ WENO_FX Limb speed(double A, int a) {
 WENO_FX i64 times_speed(const Limb &A, i64 w) {
   Acc v = {0, 0};
   mac(v, A, limb(w));
-  return acc_value(v);
+  return over63(v);
 }
 
 // The left eigenvectors of a face in the form project4 (NC = 4) and project3
 // (NC = 3) apply them: with z = b2 r - t2 m_n - t3 m_t + b1 E and
 // tc = t1 r - ic m_n the fields are z + tc, r - z, (m_t - ut r,) z - tc.
-// um: the scale of z, tc and r, projected values are x 2^(1592 - um) (below
-// 2^61.6); ut: that of m_t - ut r.  emax: the largest exponent among the
+// um: the scale of z, tc and r, projected values are x 2^(1592 - um), a field
+// below 2^61.6; us: that of m_t - ut r.  emax: the largest exponent among the
 // coefficients (2047: not finite).
 template <int NC>
 struct LeftRows {
@@ -361,11 +365,11 @@ WENO_FX LeftRows<NC> left_rows(const int (&E)[NC], double b2, double b1, double 
   o.tn = coefficient(-ic, E[1], o.um);
   return o;
 }
-// A difference vector's projections: z, tc, r (and s = m_t - ut r) from its
-// packed components v[q], with a = 0 for states, the speeds' exponent for
-// physical fluxes.
+// A difference vector's projections from its packed components v[q], with
+// a = 0 for states, the speeds' exponent for physical fluxes: z, tc and r, and
+// apart (it lives no longer than its own field) s = m_t - ut r.
 struct Proj {
-  i64 z, tc, r, s;
+  i64 z, tc, r;
 };
 template <int NC>
 WENO_FX Proj project(const LeftRows<NC> &c, const int (&E)[NC], int a, const u64 (&v)[NC]) {
@@ -379,17 +383,12 @@ WENO_FX Proj project(const LeftRows<NC> &c, const int (&E)[NC], int a, const u64
   mac(z, c.zE, d[NC - 1]);
   mac(t, c.tr, d[0]);
   mac(t, c.tn, d[1]);
-  Proj o;
-  o.z = acc_value(z);
-  o.tc = acc_value(t);
-  o.r = packed_value(v[0], c.um + a - 1018 - packed_exponent(v[0]));
-  o.s = 0;
-  if (NC == 4) {
-    Acc u = {0, 0};
-    mac(u, c.sr, d[0]);
-    o.s = acc_value(u) + packed_value(v[2], c.us + a - 1018 - packed_exponent(v[2]));
-  }
-  return o;
+  return Proj{over63(z), over63(t), packed_value(v[0], c.um + a - 1018 - packed_exponent(v[0]))};
+}
+WENO_FX i64 project_shear(const LeftRows<4> &c, const int (&E)[4], int a, u64 rho, u64 mt) {
+  Acc u = {0, 0};
+  mac(u, c.sr, limb(packed_value(rho, E[0] + a + 2 - packed_exponent(rho))));
+  return over63(u) + packed_value(mt, c.us + a - 1018 - packed_exponent(mt));
 }
 
 // The stencil differences g + x of f^+ become those of the mirrored f^-:
@@ -453,19 +452,20 @@ WENO_FX float rcpf(float x) {
 //   c = rm + sum_k D_k G_k (r_k - rm) / (20 + sum_k D_k G_k), G_k = T / b_k,
 // the second term is far below a unit, or a few units, wherever the stencil
 // resolves its data (G is the eighth power of the phase per cell, r_k - rm its
-// third): computed in FP32 on the exact second and fifth differences, with an
-// error below 2^-21 of max G max |r_k - rm|, it is good to half a unit where
-// that product is at most 2^20 units, from about 70 cells a wavelength on.
-// Returns whether it is, and the term in units.
-// SENS: a sensitivity term would lower G; the term then has to vanish (at
-// most half a unit).
+// third).  Computed in FP32 on the exact second differences and their exact
+// differences, with an error below 2^-21 of max G max |r_k - rm|, it is good
+// to 2 units (2^-58 of the bound on the projected differences) where that
+// product is at most 2^22 units, from about 70 cells a wavelength on.
+// |d_j| < 2^61: a field's differences over 4.  Returns whether it is, and the term in units.
+// SENS: a sensitivity term would lower G, so the term then has to vanish (at
+// most half a unit); without it (epsilon <= 2^-126) the same holds unless
+// every b_k is above 2^18 units squared, 2^25 times what it could be.
 template <bool SENS>
 WENO_FX bool smooth_term(const i64 (&d)[5], int &corr) {
   const i64 s0 = d[1] - d[0], s1 = d[2] - d[1], s2 = d[3] - d[2], s3 = d[4] - d[3];
-  const i64 q = s1 - s2;
-  const float r5 = to_float((s3 - s0) + 3 * q);
   const float a0 = to_float(s0), a1 = to_float(s1), a2 = to_float(s2), a3 = to_float(s3);
   const float f1 = to_float(d[1]), f2 = to_float(d[2]), f3 = to_float(d[3]);
+  const float e2 = to_float(s1 - s2), r5 = ffma(3.0f, e2, to_float(s3 - s0));
   const float t0 = ffma(2.0f, f1, a0), t1 = fadd(f1, f2), t2 = ffma(2.0f, f2, -a2),
               t3 = ffma(3.0f, a3, fmul(-2.0f, f3));
   const float b0 = ffma(fmul(13.0f, a0), a0, fmul(fmul(3.0f, t0), t0));
@@ -477,27 +477,34 @@ WENO_FX bool smooth_term(const i64 (&d)[5], int &corr) {
   const float g0 = fmul(T, rcpf(fadd(b0, tiny))), g1 = fmul(T9, rcpf(fadd(b1, tiny)));
   const float g2 = fmul(T9, rcpf(fadd(b2, tiny))), g3 = fmul(T, rcpf(fadd(b3, tiny)));
   // r_k - r_1, their mean m, and r_k - rm
-  const float e0 = fmul(2.0f, to_float(s0 - s1)), e2 = to_float(q);
+  const float e0 = fmul(2.0f, to_float(s0 - s1));
   const float e3 = ffma(2.0f, to_float(s3 - s2), e2);
   const float m = fmul(0.05f, ffma(9.0f, e2, fadd(e0, e3)));
   const float h0 = fadd(e0, -m), h2 = fadd(e2, -m), h3 = fadd(e3, -m);
   const float gs = fadd(fadd(g0, g1), fadd(g2, g3));  // 20 times a mean of the G_k
   const float hm = fmaxf(fmaxf(fabsf(h0), fabsf(h2)), fmaxf(fabsf(h3), fabsf(m)));
+  const float most = fmul(gs, hm);
+  if (SENS) {
+    corr = 0;
+    return most <= 8 * 0x1p-32f;
+  }
   const float c = fmul(ffma(g0, h0, ffma(g2, h2, ffma(g3, h3, -fmul(g1, m)))),
                        rcpf(fadd(20.0f, gs)));
-  const bool ok = fmul(gs, hm) <= (SENS ? 8 * 0x1p-32f : 16 * 0x1p-12f);
-  corr = (SENS || !ok) ? 0 : (int)ffma(c, 0x1p32f, c < 0.0f ? -0.5f : 0.5f);
+  const bool ok = most <= 16 * 0x1p-10f &&
+                  (most <= 8 * 0x1p-32f || fminf(fminf(b0, b1), fminf(b2, b3)) >= 0x1p-46f);
+  corr = ok ? (int)ffma(c, 0x1p32f, c < 0.0f ? -0.5f : 0.5f) : 0;
   return ok;
 }
 
 // c^+ + c^- less 6 alpha dw_2 of a smooth field: the linear parts add up to
 // (7 (g_1 - g_3) - (g_0 - g_4)) / 5 (alpha drops out of the central flux).
+// In units of 4, as the terms.
 WENO_FX i64 smooth_sum(const i64 (&g)[5], int corr) {
-  const i64 v = 7 * (g[1] - g[3]) - (g[0] - g[4]);  // below 2^63
-  // v / 5 = (v >> 32) 2^32 / 5 + ..: 2^63 / 5 in two limbs
-  Acc p = {0, 0};
-  mac(p, Limb{0x19999999, 0x4CCCCCCD}, limb(v));
-  return (p.hi << 1) + (p.cr >> 30) + corr;
+  const i64 v = (g[1] >> 2) - (g[3] >> 2);
+  const i64 u = 2 * v - ((g[0] >> 2) - (g[4] >> 2));  // v + u / 5
+  Acc p = {0, 0};  // u times 2^63 / 5
+  mac(p, Limb{0x19999999, 0x4CCCCCCD}, limb(u));
+  return v + over63(p) + corr;
 }
 
 // c^+ + c^- less 6 alpha dw_2 by the weights, one flux after the other.
@@ -513,6 +520,16 @@ WENO_FX i64 rough_sum(i64 (&x)[5], i64 (&g)[5], Recon recon) {
     mirror(x, g);
   }
   return S;
+}
+
+// S 2^k, rounded to nearest, by shifts (a conversion from a 64-bit integer
+// issues to the FP64 pipe).
+WENO_FX double from_fixed(i64 S, int k) {
+  const u64 a = abs64(S);
+  const int n = clz64(a);
+  const u64 v = shl(a, n), r = (v >> 11) + ((v >> 10) & 1);  // the leading bit adds to the exponent
+  const u64 b = r + ((u64)(i64)(1085 + k - n) << 52);
+  return bitsd(S == 0 ? 0 : (S < 0 ? b | 0x8000000000000000ull : b));
 }
 
 // 2^k / 6 for -1019 <= k <= 1026.

@@ -5,6 +5,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "weno_fixed.cuh"
+
 #ifdef __CUDACC__
 #define WENO_HD __host__ __device__
 #else
@@ -40,6 +42,39 @@ WENO_HD constexpr bool all_tile_shapes(int mode, bool p1, int precision) {
 WENO_HD constexpr int tile_shape_built(bool all, int v) {
   return all ? v : (v == 8 ? 8 : (v == 2 || v == 4 || v == 7 ? 2 : 9));
 }
+
+// Parameters of eqs. (21)-(22) for one characteristic field.  The field's
+// split fluxes reach the reconstruction multiplied by `scale` (2 or 4, see
+// the projection below), so mu_0 and, without Ai, epsilon are scaled to keep
+// Gamma_k exactly the paper's.
+struct ReconParams {
+  double eps4;   // 4 * eps            (indicators are carried as 4*beta, 4*tau)
+  double mu0s;   // scale * mu_0       (Ai)
+  double efix;   // 4 * eps * scale^2  (no Ai: mu = 1)
+  double p;      // power parameter of eq. (21)
+  double me;     // sqrt(4 eps) / 6    (Ai: 4 eps mu^2 = (me * dev + mo)^2, dev =
+  double mo;     // sqrt(4 eps) * scale * mu_0   the sum of |v_j - mean v|)
+  double e0;     // mo^2: the term of a flat stencil (dev = 0)
+  float mef;     // me^2 = eps / 9 = mef 2^eme, mef in [1, 2) (FP32)
+  int eme;
+  int lthr;      // dev >= 2^(lthr - 1019) implies me dev >= 2^30 mo (mo negligible)
+  int es_lo, es_hi;  // exponents of a field's largest difference the integer path takes
+  fx::Flt e3;        // 3 efix (no Ai), in the data's units squared
+};
+// FP32 reconstruction (za6_f32).
+struct Recon32 {
+  float eps4;   // 4 * eps32
+  float p;      // power parameter
+};
+// The scheme's constants for fields of scale 2 and 4.  Formed on the host: one
+// thread a block forming them (a square root and ~100 FP64 operations on a pipe
+// that takes 64 clocks a warp) kept every block waiting for microseconds.
+struct SchemeParams {
+  ReconParams rp[2];
+  Recon32 r32;
+  double rdx, rdy;  // 1/dx, 1/dy
+};
+SchemeParams scheme_params(double eps, double mu0, double p, bool ai, double dx, double dy);
 
 // Everything one stage launch needs (passed by value).
 struct StageArgs {
@@ -79,6 +114,9 @@ struct StageArgs {
   // output's first / last r rows are copied into send_lo / send_hi (same layout).
   const double *halo_lo, *halo_hi;
   double *send_lo, *send_hi;
+  // the scheme's constants (set by launch_stage; of a slot, in the engine)
+  SchemeParams sp;
+  const SchemeParams *sp_at;  // where they are, NULL: sp
   // set by the 2D launcher: interior tiles stage by TMA through the tensor
   // map passed beside these arguments; tma_no_copy (a test of the bounded
   // wait, WENO_TEST_TMA_NO_COPY=1 in the environment) arms the barrier but
@@ -104,6 +142,7 @@ struct SlotDev {
   int ndim, nc, bc_x, bc_y, precision, alpha_single, active, pad;
   long long nx, ny;
   double dx, dy, gamma, cfl, eps, mu0, p, t_final;
+  SchemeParams sp;
   double *U, *U1, *U2;          // state and the two stage buffers
   unsigned long long *alpha;    // [3][8] rotating speed-maxima slots
   double *clock;                // t, tnext, dt

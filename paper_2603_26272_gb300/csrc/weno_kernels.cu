@@ -2,6 +2,10 @@
 // persistent stage kernel and the host-side launchers for GB300 (sm_103a).
 // The tile kernels themselves are in weno_tiles.cuh, instantiated by weight
 // mode in weno_stage_*.cu (sixth order) and by order in weno_orders.cu.
+#include <algorithm>
+#include <cfloat>
+#include <cmath>
+#include <cstring>
 #include <mutex>
 
 #include "weno_tiles.cuh"
@@ -33,13 +37,21 @@ __global__ void __launch_bounds__(256) k_alpha(const AlphaArgs a) {
   }
   const double gm1 = a.gamma - 1.0;
   unsigned long long vm[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
-  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < plane;
-       k += (long long)gridDim.x * blockDim.x) {
+  // After the first round the maxima so far, of every block, are floors below
+  // which a cell needs no FP64 speeds (2D; speeds_below): at 2048^2 the pass
+  // was bound by FP64 issue (258 us for 134 MB).
+  const float gg = (float)(a.gamma * gm1);
+  float floors[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  const bool filter = a.nc == 4 && plane > 2 * stride;
+  bool first = filter;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < plane; k += stride) {
     const double rho = Ub[k];
-    const double ir = rcp_pos(rho);
     const double mx = Ub[plane + k];
     const double my = (a.nc == 4) ? Ub[2 * plane + k] : 0.0;
     const double E = Ub[(a.nc - 1) * plane + k];
+    if (filter && !first && speeds_below(rho, mx, my, E, gg, floors)) continue;
+    const double ir = rcp_pos(rho);
     const double u = mx * ir, v = my * ir;
     const double p = gm1 * (E - 0.5 * fma(mx, u, my * v));
     if (!(pos_finite(rho) && pos_finite(p)))
@@ -51,7 +63,18 @@ __global__ void __launch_bounds__(256) k_alpha(const AlphaArgs a) {
     vm[3] = max(vm[3], abs_bits(v - cs));
     vm[4] = max(vm[4], abs_bits(v));
     vm[5] = max(vm[5], abs_bits(v + cs));
+    if (first) {  // every thread of the grid has a first cell (plane > 2 stride)
+      first = false;
+      const int slot[6] = {0, 1, 3, 4, 5, 7};
+      const int dup[6] = {-1, 2, -1, -1, 6, -1};
+      unsigned long long w[6] = {vm[0], vm[1], vm[2], vm[3], vm[4], vm[5]};
+      block_max_atomic<6>(w, a.alpha_out + b * 8, slot, dup);
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < 6; ++q) floors[q] = speed_floor(a.alpha_out + b * 8, q);
+    }
   }
+  __syncthreads();
   if (a.nc == 3) {
     const int slot[6] = {0, 1, 2, 4, 5, 7};  // 1D: fields u-c, u, u+c in slots 0..2
     const int dup[6] = {-1, -1, -1, -1, -1, -1};
@@ -146,6 +169,7 @@ __device__ __forceinline__ StageArgs slot_stage_args(const SlotDev &S, int stage
   a.halo_lo = a.halo_hi = nullptr;
   a.send_lo = a.send_hi = nullptr;
   a.use_tma = a.tma_no_copy = 0;
+  a.sp_at = &S.sp;
   a.t = S.clock;
   a.tnext = S.clock + 1;
   a.dt = S.clock + 2;
@@ -238,7 +262,62 @@ bool encode_state_map(const double *U, long long nbatch, long long ny, long long
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-cudaError_t launch_stage(const StageArgs &a, cudaStream_t s) {
+// The scheme's constants for a field that arrives scaled by k.
+static ReconParams recon_params(double eps, double mu0, double p, bool ai, double k) {
+  auto bits = [](double x) {
+    unsigned long long b;
+    std::memcpy(&b, &x, 8);
+    return b;
+  };
+  ReconParams r;
+  std::memset(&r, 0, sizeof(r));
+  r.eps4 = 4.0 * eps;
+  r.mu0s = k * mu0;
+  r.efix = 4.0 * eps * k * k;
+  r.p = p;
+  const double se = std::sqrt(4.0 * eps);
+  r.me = se * (1.0 / 6.0);
+  r.mo = se * (k * mu0);
+  r.e0 = r.mo * r.mo;
+  // me^2 = eps / 9 as an FP32 mantissa and an exponent (eps / 9 is a normal
+  // double for every eps the boundary accepts with Ai)
+  const unsigned long long b2 = bits(eps * (1.0 / 9.0));
+  r.eme = (int)((b2 >> 52) & 0x7FF) - 1023;
+  const unsigned mb = 0x3F800000u | (unsigned)((b2 >> 29) & 0x7FFFFFu);
+  std::memcpy(&r.mef, &mb, 4);
+  // dev >= 2^(lthr - 1019) implies dev / 6 >= 2^30 scale mu_0: with
+  // 6 scale mu_0 < 2^(E + 1), E its exponent, lthr = 1019 + E + 1 + 30
+  r.lthr = mu0 > 0.0 ? 1019 + ((int)((bits(6.0 * k * mu0) >> 52) & 0x7FF) - 1023) + 31 : -(1 << 20);
+  // the integer path: exponents from 64 up (to_fixed) and, where it leaves the
+  // sensitivity term out, from a largest difference of scale mu_0 up; squares
+  // of differences up to 2^400 in the sensitivity term's FP64
+  const bool tiny = weight_mode(ai, eps, mu0) == kAiTiny;
+  r.es_hi = tiny ? 2046 : 1023 + 400;
+  r.es_lo = 64;
+  if (tiny) r.es_lo = std::max(64, (int)((bits(k * mu0) >> 52) & 0x7FF) + 1);
+  const unsigned long long b3 = bits(std::fmax(3.0 * r.efix, DBL_MIN));
+  r.e3.m = (b3 << 11) | 0x8000000000000000ull;
+  r.e3.e = (int)(b3 >> 52) - 1086;
+  if (!tiny && (b3 >> 52) >= 2047) r.es_lo = 4096;
+  return r;
+}
+
+SchemeParams scheme_params(double eps, double mu0, double p, bool ai, double dx, double dy) {
+  SchemeParams s;
+  std::memset(&s, 0, sizeof(s));
+  s.rp[0] = recon_params(eps, mu0, p, ai, 2.0);
+  s.rp[1] = recon_params(eps, mu0, p, ai, 4.0);
+  s.r32.eps4 = 4.0e-30f;
+  s.r32.p = (float)p;
+  s.rdx = 1.0 / dx;
+  s.rdy = 1.0 / dy;
+  return s;
+}
+
+cudaError_t launch_stage(const StageArgs &a_in, cudaStream_t s) {
+  StageArgs a = a_in;
+  a.sp = scheme_params(a.eps, a.mu0, a.p, a.ai != 0, a.dx, a.dy);
+  a.sp_at = nullptr;
   if (a.order_r != 3) return launch_stage_orders(a, s);  // weno_orders.cu
   if (a.precision == 1) return launch_stage_fp32(a, s);
   const int mode = weight_mode(a.ai != 0, a.eps, a.mu0);

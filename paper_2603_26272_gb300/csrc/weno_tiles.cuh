@@ -133,52 +133,16 @@ __device__ bool stage_control(const StageArgs &a, long long b, bool first_block_
   return s_go != 0;
 }
 
-// Per-field reconstruction parameters; field m arrives scaled by k[m].
-__device__ __forceinline__ ReconParams make_rp(const StageArgs &a, double k) {
-  ReconParams r;
-  r.eps4 = 4.0 * a.eps;
-  r.mu0s = k * a.mu0;
-  r.efix = 4.0 * a.eps * k * k;
-  r.p = a.p;
-  const double se = sqrt(4.0 * a.eps);
-  r.me = se * (1.0 / 6.0);
-  r.mo = se * (k * a.mu0);
-  r.e0 = r.mo * r.mo;
-  // me^2 = eps / 9 as an FP32 mantissa and an exponent (eps / 9 is a normal
-  // double for every eps the boundary accepts with Ai)
-  const double me2 = a.eps * (1.0 / 9.0);
-  const int hi = __double2hiint(me2);
-  r.eme = ((hi >> 20) & 0x7FF) - 1023;
-  r.mef = __uint_as_float(0x3F800000u |
-                          (__funnelshift_r((unsigned)__double2loint(me2), (unsigned)hi, 29) & 0x7FFFFFu));
-  // dev >= 2^(lthr - 1019) implies dev / 6 >= 2^30 scale mu_0: with
-  // 6 scale mu_0 < 2^(E + 1), E its exponent, lthr = 1019 + E + 1 + 30
-  if (a.mu0 > 0.0) {
-    const double m6 = 6.0 * k * a.mu0;
-    r.lthr = 1019 + (((__double2hiint(m6) >> 20) & 0x7FF) - 1023) + 31;
-  } else {
-    r.lthr = -(1 << 20);
-  }
-  // the integer path: exponents from 64 up (to_fixed) and, where it leaves the
-  // sensitivity term out, from a largest difference of scale mu_0 up; squares
-  // of differences up to 2^400 in the sensitivity term's FP64
-  const bool tiny = a.ai && a.eps <= 0x1p-126 && a.mu0 <= 0x1p-100;
-  r.es_hi = tiny ? 2046 : 1023 + 400;
-  r.es_lo = 64;
-  if (tiny) r.es_lo = max(64, ((__double2hiint(k * a.mu0) >> 20) & 0x7FF) + 1);
-  const double e3 = fmax(3.0 * r.efix, DBL_MIN);
-  const unsigned long long b = (unsigned long long)__double_as_longlong(e3);
-  r.e3.m = (b << 11) | 0x8000000000000000ull;
-  r.e3.e = (int)(b >> 52) - 1086;
-  if (!tiny && (b >> 52) >= 2047) r.es_lo = 4096;
-  return r;
+// The scheme's constants into shared memory (published by the caller's next
+// barrier).
+__device__ __forceinline__ const SchemeParams &scheme_of(const StageArgs &a) {
+  return a.sp_at ? *a.sp_at : a.sp;
 }
-
-__device__ __forceinline__ Recon32 make_r32(const StageArgs &a) {
-  Recon32 r;
-  r.eps4 = 4.0e-30f;
-  r.p = (float)a.p;
-  return r;
+__device__ __forceinline__ void load_scheme(const StageArgs &a, SchemeParams &s) {
+  static_assert(sizeof(SchemeParams) % 8 == 0, "copied as doubles");
+  const double *const src = reinterpret_cast<const double *>(&scheme_of(a));
+  for (int k = threadIdx.x; k < (int)(sizeof(SchemeParams) / 8); k += blockDim.x)
+    reinterpret_cast<double *>(&s)[k] = src[k];
 }
 
 // Block reduction of NV maxima (bit patterns) and one atomicMax per value into
@@ -324,8 +288,37 @@ __device__ __forceinline__ void cell_source(const StageArgs &a, const double *Ub
   }
 }
 
+// The speed maxima of eq. (6) are exact, but most cells are far from setting
+// one: a cell whose FP32 estimates stay below what the six maxima have already
+// reached needs no FP64 speeds (22 FP64 operations, a tenth of a stage's).
+// Floors: the next stage's slot as it stands (any earlier value is a lower
+// bound of the final maximum).
+__device__ __forceinline__ constexpr int speed_slot(int q) {  // |u-c|, |u|, |u+c|, |v-c|, |v|, |v+c|
+  return q == 0 ? 0 : (q == 1 ? 1 : (q == 2 ? 3 : (q == 3 ? 4 : (q == 4 ? 5 : 7))));
+}
+__device__ __forceinline__ float speed_floor(const unsigned long long *slot, int q) {
+  return f32_rn(bits2d(__ldcg(slot + speed_slot(q))));
+}
+// True where the state is physical and none of its speeds can reach its floor,
+// with a margin of 2^-9 of the speeds for the FP32 arithmetic (p above 2^-12 E,
+// so the sound speed is good to 2^-11); false (FP64 decides) for anything else,
+// NaN and magnitudes near FP32's limits included.
+__device__ __forceinline__ bool speeds_below(double rho, double mx, double my, double E, float gg,
+                                             const float *floors) {
+  const float r = f32_rn(rho), m = f32_rn(mx), n = f32_rn(my), e = f32_rn(E);
+  const float ir = fx::rcpf(r), u = m * ir, v = n * ir;
+  const float pe = e - 0.5f * (m * u + n * v);
+  if (!(r > 1e-18f && r < 1e18f && e > 1e-18f && e < 1e18f && pe > e * 0x1p-12f)) return false;
+  float c;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(gg * pe * ir));
+  const float mg = 0x1p-9f * (fmaxf(fabsf(u), fabsf(v)) + c);
+  return fabsf(u - c) + mg < floors[0] && fabsf(u) + mg < floors[1] &&
+         fabsf(u + c) + mg < floors[2] && fabsf(v - c) + mg < floors[3] &&
+         fabsf(v) + mg < floors[4] && fabsf(v + c) + mg < floors[5];
+}
+
 // Phase 3 of a 2D tile: per cell the conservative difference of eq. (5)
-// from the faces' 4 F (backproject4, so idx = 0.25 / dx, idy = 0.25 / dy), the
+// from the faces' multiples of F (the factor goes with idx, idy), the
 // Runge-Kutta combination with the staged input u_at(r, c, q) of tile cell
 // (r, c), the strips' send rows, and the next stage's speed maxima.
 template <int TX, int TY, int R, class UAt>
@@ -338,6 +331,12 @@ __device__ __forceinline__ void tile2d_update(const StageArgs &a, long long b, l
   const int tid = threadIdx.x;
   unsigned long long mx6[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
   const bool want_alpha = (a.mode == 0) && (a.alpha_out != nullptr);
+  const float gg = (float)(a.gamma * gm1);
+  __shared__ float floors[6];
+  if (want_alpha) {
+    if (tid < 6) floors[tid] = speed_floor(a.alpha_out + b * 8, tid);
+    __syncthreads();
+  }
   for (int k = tid; k < TX * TY; k += blockDim.x) {
     const int r = k / TX, c = k - r * TX;
     const long long gi = i0 + c, gj = j0 + r;
@@ -365,7 +364,7 @@ __device__ __forceinline__ void tile2d_update(const StageArgs &a, long long b, l
     if (a.send_hi && gj >= a.ny - R)
 #pragma unroll
       for (int q = 0; q < 4; ++q) a.send_hi[((b * 4 + q) * R + (gj - (a.ny - R))) * a.nx + gi] = uo[q];
-    if (want_alpha) {
+    if (want_alpha && !speeds_below(uo[0], uo[1], uo[2], uo[3], gg, floors)) {
       const double ir = rcp_pos(uo[0]);
       const double u = uo[1] * ir, v = uo[2] * ir;
       const double p = gm1 * (uo[3] - 0.5 * fma(uo[1], u, uo[2] * v));
@@ -427,6 +426,15 @@ __host__ __device__ constexpr size_t smem_euler2d_tma() {
   return R == 3 ? Tile6<TX, TY>::kBytes
                 : ((smem_euler2d_gen<TX, TY, R>() + 127) & ~size_t(127)) +
                       tma_box_bytes<TX, TY, R>() + 128;
+}
+
+// GLF speed of field m of nc (max|u| + c for every field in the single mode).
+__device__ __forceinline__ double field_speed(const StageArgs &a, const unsigned long long *al,
+                                              int m, int nc) {
+  unsigned long long v = al[m];
+  if (a.alpha_single)
+    for (int q = 0; q < nc; ++q) v = max(v, al[q]);
+  return bits2d(v);
 }
 
 // One tile (tile index `tile` of problem b) of a 2D stage, run by one block.
@@ -504,7 +512,7 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
   // Phase 2: every x- and y-face of the tile once.  Lanes of a warp may mix
   // directions; the code path is the same (only the plane indices differ).
   const unsigned long long *al = a.alpha_in + b * 8;
-  const ReconParams rp4 = make_rp(a, 4.0), rp2 = make_rp(a, 2.0);
+  const ReconParams rp4 = a.sp.rp[1], rp2 = a.sp.rp[0];
   for (int f = tid; f < NFX + NFY; f += blockDim.x) {
     int base, stride, dir, fr, fc;
     if (f < NFX) {
@@ -528,12 +536,8 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
                   pl[7 * REG + kR], pl[pun * REG + kR], pl[put * REG + kR], pl[6 * REG + kR],
                   gm1, fs))
       record_status(a.status, 3, a.stage, b, j0 + (dir ? fr : fr), i0 + fc);
-    double A1 = bits2d(al[4 * dir + 0]), A2 = bits2d(al[4 * dir + 1]);
-    double A3 = bits2d(al[4 * dir + 2]), A4 = bits2d(al[4 * dir + 3]);
-    if (a.alpha_single) {
-      const double m = fmax(fmax(A1, A2), fmax(A3, A4));
-      A1 = A2 = A3 = A4 = m;
-    }
+    const double A1 = field_speed(a, al + 4 * dir, 0, 4), A2 = field_speed(a, al + 4 * dir, 1, 4);
+    const double A3 = field_speed(a, al + 4 * dir, 2, 4), A4 = field_speed(a, al + 4 * dir, 3, 4);
     double h1, h2, h3, h4;
     {
       // f^+ in stencil order, f^- mirrored (its upwind side is on the right).
@@ -569,7 +573,7 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
   }
   __syncthreads();
 
-  tile2d_update<TX, TY, R>(a, b, i0, j0, dt, fx, fy, 0.25 / a.dx, 0.25 / a.dy,
+  tile2d_update<TX, TY, R>(a, b, i0, j0, dt, fx, fy, 0.25 * a.sp.rdx, 0.25 * a.sp.rdy,
                            [&](int r, int c, int q) { return pl[q * REG + (R + r) * W + R + c]; });
 }
 
@@ -602,15 +606,6 @@ __device__ __forceinline__ void normal_flux(double rho, double mn, double mt, do
   F1 = fma(mn, un, p);
   F2 = mt * un;
   F3 = H * mn;
-}
-
-// GLF speed of field m of nc (max|u| + c for every field in the single mode).
-__device__ __forceinline__ double field_speed(const StageArgs &a, const unsigned long long *al,
-                                              int m, int nc) {
-  unsigned long long v = al[m];
-  if (a.alpha_single)
-    for (int q = 0; q < nc; ++q) v = max(v, al[q]);
-  return bits2d(v);
 }
 
 // The GLF speeds of a problem in fixed point, per direction (fx::speed), and
@@ -672,8 +667,7 @@ __device__ __noinline__ double face_wide(const double *sm, int dir, int fr, int 
 template <int TX, int TY, int AI, bool P1, int PREC>
 __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long long b, long long i0,
                                             long long j0, double gm1, double *sm,
-                                            const ReconParams &rp2, const ReconParams &rp4,
-                                            const Speeds &sp) {
+                                            const SchemeParams &scheme, const Speeds &sp) {
   using L = Tile6<TX, TY>;
   constexpr int R = 3, W = L::W, BW = L::BW, XO = L::XO, PB = L::PB, REG = L::REG, ND = L::ND;
   const double *const box = sm + L::kBox;
@@ -730,7 +724,7 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long lo
   const int NF = dir ? L::NFY : L::NFX, lf = dir ? TX : TX + 1, jf = dir ? inv(TX) : inv(TX + 1);
   const int ps = dir ? TX : 1;  // pair stride along the stencil
   const unsigned long long *al = a.alpha_in + b * 8 + 4 * dir;
-  const Recon32 r32 = make_r32(a);
+  const ReconParams &rp2 = scheme.rp[0], &rp4 = scheme.rp[1];
   for (int f = tid; f < NF; f += blockDim.x) {
     const int fr = rows_of(f, jf), fc = f - fr * lf;
     const int p0 = fr * lp + fc;
@@ -745,8 +739,8 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long lo
     if constexpr (kPacked) {
       const fx::u64 *const pf = dp + p0;
       face_fields<4, AI>(
-          fs, sp.ka[dir], sp.ea[dir], [&](int q, int j) { return pf[q * ND + j * ps]; },
-          [&](int q, int j) { return pf[(q == 0 ? 1 : 3 + q) * ND + j * ps]; },
+          fs, sp.ka[dir], sp.ea[dir],
+          [&](int s, int q, int j) { return pf[(s ? (q == 0 ? 1 : 3 + q) : q) * ND + j * ps]; },
           [&](int m) -> const ReconParams & { return (m == 0 || m == 3) ? rp4 : rp2; },
           [&](int m) {
             return face_wide<TX, TY, AI>(sm, dir, fr, fc, m, fs.un, fs.ut, fs.ic, fs.b1, fs.b2,
@@ -768,15 +762,16 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long lo
       for (int m = 0; m < 4; ++m) {
         const double A = field_speed(a, al, m, 4);
         if constexpr (PREC == 1)
-          h[m] = field_flux_f32d<P1>(dw[m], dg[m], A, r32);
+          h[m] = field_flux_f32d<P1>(dw[m], dg[m], A, scheme.r32);
         else
           h[m] = field_flux<AI, P1>(dw[m], dg[m], A, (m == 0 || m == 3) ? rp4 : rp2, 0.0);
       }
     }
     double F0, F1, F2, F3;
     backproject4(fs, h[0], h[1], h[2], h[3], F0, F1, F2, F3);
-    // the centre values: 4 F_hat += 2 (F_L + F_R) (= 4 F_L + 2 dF of the centre
-    // pair, where the differences are staged in FP64)
+    // the centre values.  Packed: the faces hold 2 F_hat, F_L + F_R and a twelfth
+    // of what backproject4 gives from the fields' 6 h; else 4 F_hat, with
+    // 2 (F_L + F_R) = 4 F_L + 2 dF of the centre pair.
     {
       const double mnL = bn[oL];
       double FL1, FL2, FL3;
@@ -786,10 +781,10 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long lo
         double FR1, FR2, FR3;
         normal_flux(box[oR], mnR, bt[oR], box[3 * PB + oR], un[kR], pl[3 * REG + kR], FR1, FR2,
                     FR3);
-        F0 = fma(2.0, mnL + mnR, F0);
-        F1 = fma(2.0, FL1 + FR1, F1);
-        F2 = fma(2.0, FL2 + FR2, F2);
-        F3 = fma(2.0, FL3 + FR3, F3);
+        F0 = fma(1.0 / 12.0, F0, mnL + mnR);
+        F1 = fma(1.0 / 12.0, F1, FL1 + FR1);
+        F2 = fma(1.0 / 12.0, F2, FL2 + FR2);
+        F3 = fma(1.0 / 12.0, F3, FL3 + FR3);
       } else {
         const int pc = p0 + 2 * ps;
         F0 = fma(4.0, mnL, fma(2.0, dd[ND + pc], F0));
@@ -830,16 +825,9 @@ __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, l
   const double gm1 = a.gamma - 1.0;
   const int tid = threadIdx.x;
 
-  // per-block constants (published by the barrier after phase 1): the
-  // reconstruction parameters of the field scales 2 and 4, 0.25 / dx, dy
-  __shared__ ReconParams s_rp[2];
-  __shared__ double s_id[2];
-  if (tid == 0) {
-    s_rp[0] = make_rp(a, 2.0);
-    s_rp[1] = make_rp(a, 4.0);
-    s_id[0] = 0.25 / a.dx;
-    s_id[1] = 0.25 / a.dy;
-  }
+  // the scheme's constants and speeds (published by the barrier after phase 1)
+  __shared__ SchemeParams s_scheme;
+  load_scheme(a, s_scheme);
   __shared__ Speeds s_sp;
   make_speeds(a, b, 4, s_sp);
 
@@ -891,9 +879,11 @@ __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, l
 
 #pragma unroll 1
   for (int dir = 0; dir < 2; ++dir)
-    tile6_sweep<TX, TY, AI, P1, PREC>(a, dir, b, i0, j0, gm1, sm, s_rp[0], s_rp[1], s_sp);
+    tile6_sweep<TX, TY, AI, P1, PREC>(a, dir, b, i0, j0, gm1, sm, s_scheme, s_sp);
 
-  tile2d_update<TX, TY, R>(a, b, i0, j0, dt, sm + L::kFx, sm + L::kFy, s_id[0], s_id[1],
+  constexpr double f = P1 && PREC == 0 ? 0.5 : 0.25;  // the faces hold 2 F or 4 F
+  tile2d_update<TX, TY, R>(a, b, i0, j0, dt, sm + L::kFx, sm + L::kFy, f * s_scheme.rdx,
+                           f * s_scheme.rdy,
                            [&](int r, int c, int q) { return box[q * PB + (R + r) * BW + XO + c]; });
 }
 
@@ -913,7 +903,7 @@ __device__ __forceinline__ void euler2d_tile(const StageArgs &a, long long b, lo
 // tm: tensor map of a.Uin (see euler2d_tile), used when a.use_tma is set.
 template <int TX, int TY, int NT, int MINB, int AI, bool P1, int PREC, int R = 3>
 __global__ void __launch_bounds__(NT, MINB)
-    k_euler2d(const StageArgs a, const __grid_constant__ CUtensorMap tm) {
+    k_euler2d(const __grid_constant__ StageArgs a, const __grid_constant__ CUtensorMap tm) {
   extern __shared__ __align__(128) double sm[];
   euler2d_tile<TX, TY, AI, P1, PREC, R>(a, blockIdx.z, blockIdx.x,
                                         blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, sm,

@@ -1,7 +1,7 @@
 // weno_tiles1d.cuh -- the 1D stage kernels (Euler and scalar equations) of
 // the central-upwind WENO right-hand side, templated on the stencil
 // half-width r.  Included by weno_tiles.cuh inside its namespaces; it uses
-// the helpers defined there (stage_control, make_rp, block_max_atomic, ...).
+// the helpers defined there (stage_control, load_scheme, block_max_atomic, ...).
 #pragma once
 
 // ---------------------------------------------------------------------------
@@ -14,8 +14,9 @@
 // after the back-projection.
 // ---------------------------------------------------------------------------
 // The centre values of a sixth-order 1D Euler face between cells L and L+1 of
-// the staged fluxes pl[6..8]: 4 F_hat += 2 (F_L + F_{L+1}) (R L = I), as
-// 4 F_L + 2 dF of pair L where the differences dd are staged in FP64.
+// the staged fluxes pl[6..8] (R L = I).  With dd, FP64 differences:
+// 4 F_hat += 4 F_L + 2 dF of pair L; without, from the fields' 6 h: the face
+// gets 2 F_hat, F_L + F_{L+1} and a twelfth of what backproject3 gives.
 template <int REG>
 __device__ __forceinline__ void add_centre3(const double (*pl)[REG], const double *dd, int nd,
                                             int L, double &F0, double &F1, double &F2) {
@@ -24,9 +25,9 @@ __device__ __forceinline__ void add_centre3(const double (*pl)[REG], const doubl
     F1 = fma(4.0, pl[7][L], fma(2.0, dd[3 * nd + L], F1));
     F2 = fma(4.0, pl[8][L], fma(2.0, dd[4 * nd + L], F2));
   } else {
-    F0 = fma(2.0, pl[6][L] + pl[6][L + 1], F0);
-    F1 = fma(2.0, pl[7][L] + pl[7][L + 1], F1);
-    F2 = fma(2.0, pl[8][L] + pl[8][L + 1], F2);
+    F0 = fma(1.0 / 12.0, F0, pl[6][L] + pl[6][L + 1]);
+    F1 = fma(1.0 / 12.0, F1, pl[7][L] + pl[7][L + 1]);
+    F2 = fma(1.0 / 12.0, F2, pl[8][L] + pl[8][L + 1]);
   }
 }
 
@@ -101,19 +102,11 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
   const double *Ub = a.Uin + b * NC * nx;
   const double gm1 = a.gamma - 1.0;
   const int tid = threadIdx.x;
-  // per-block constants, published by the barrier after the staging: the
-  // reconstruction parameters of the field scales 2 and 4, FP32 ones, and
-  // the flux difference's factor (the faces hold 4 F for Euler, 2 F for a
-  // scalar: the split without 1/2)
-  __shared__ ReconParams s_rp[2];
-  __shared__ Recon32 s_r32;
-  __shared__ double s_idx;
-  if (tid == 0) {
-    s_rp[0] = make_rp(a, 2.0);
-    s_rp[1] = make_rp(a, 4.0);
-    s_r32 = make_r32(a);
-    s_idx = (NC == 3 ? 0.25 : 0.5) / a.dx;
-  }
+  // the scheme's constants and speeds, published by the barrier after the staging
+  __shared__ SchemeParams s_scheme;
+  load_scheme(a, s_scheme);
+  const ReconParams *const s_rp = s_scheme.rp;
+  const Recon32 &s_r32 = s_scheme.r32;
   __shared__ Speeds s_sp;
   if constexpr (kPacked) make_speeds(a, b, 3, s_sp);
 
@@ -208,11 +201,12 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     if (!roe_face(pl[5][kL], pl[3][kL], 0.0, pl[4][kL], pl[5][kR], pl[3][kR], 0.0, pl[4][kR], gm1,
                   fs) && act && r == 0)
       record_status(a.status, 3, a.stage, b, 0, i0 + f);
-    auto du = [&](int c, int j) { return dp[c * ND + f + j]; };
-    auto df = [&](int c, int j) { return dp[(c == 0 ? 1 : 2 + c) * ND + f + j]; };
-    int E[3];
+    auto diff = [&](int s, int c, int j) {
+      return dp[(s ? (c == 0 ? 1 : 2 + c) : c) * ND + f + j];
+    };
+    int E[3], top;
     const int ea = s_sp.ea[0];
-    bool ok = face_exponents<3>(ea, du, df, E);
+    bool ok = face_exponents<3>(ea, diff, E, top);
     const fx::LeftRows<3> rows =
         fx::left_rows<3>(E, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic), __dmul_rn(fs.b1, fs.un),
                          __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
@@ -220,9 +214,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     fx::i64 v[5];
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-      const fx::u64 in[3] = {sgn ? dp[ND + f + j] : dp[f + j],
-                             sgn ? dp[3 * ND + f + j] : dp[ND + f + j],
-                             sgn ? dp[4 * ND + f + j] : dp[2 * ND + f + j]};
+      const fx::u64 in[3] = {diff(sgn, 0, j), diff(sgn, 1, j), diff(sgn, 2, j)};
       const fx::Proj p = fx::project<3>(rows, E, sgn ? ea : 0, in);
       v[j] = q == 1 ? p.r - p.z : (q == 0 ? p.z + p.tc : p.z - p.tc);
     }
@@ -231,8 +223,9 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     double h = field_lanes<AI>(v, s_sp.ka[0][q], rows.um + ea - 1592, ok, sgn, other, rp,
                                          wide);
     if (wide && act && sgn == 0)
-      h = face_wide3<REG, AI>(pl, f, q, fs.un, fs.ic, fs.b1, fs.b2,
-                                        field_speed(a, a.alpha_in + b * 8, q, 3), rp);
+      h = 6.0 * face_wide3<REG, AI>(
+                                     pl, f, q, fs.un, fs.ic, fs.b1, fs.b2,
+                                     field_speed(a, a.alpha_in + b * 8, q, 3), rp);
     const double h1 = __shfl_sync(0xffffffffu, h, min(lane + 1, 31)),
                  h2 = __shfl_sync(0xffffffffu, h, min(lane + 2, 31));
     if (act && r == 0) {
@@ -332,8 +325,10 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
         if constexpr (kPacked) {
           double hs[3];
           face_fields<3, AI>(
-              fs, s_sp.ka[0], s_sp.ea[0], [&](int c, int j) { return dp[c * ND + f + j]; },
-              [&](int c, int j) { return dp[(c == 0 ? 1 : 2 + c) * ND + f + j]; },
+              fs, s_sp.ka[0], s_sp.ea[0],
+              [&](int s, int c, int j) {
+                return dp[(s ? (c == 0 ? 1 : 2 + c) : c) * ND + f + j];
+              },
               [&](int m) -> const ReconParams & { return s_rp[m == 1 ? 0 : 1]; },
               [&](int m) {
                 return face_wide3<REG, AI>(pl, f, m, fs.un, fs.ic, fs.b1, fs.b2,
@@ -394,9 +389,8 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
   }
   __syncthreads();
 
-  // The faces hold 4 F (Euler, backproject3) or 2 F (a scalar: the split
-  // without 1/2), so that factor goes with 1/dx.
-  const double idx = s_idx;
+  // the faces hold 4 F for Euler off the packed path, else 2 F
+  const double idx = (NC == 3 && !kPacked ? 0.25 : 0.5) * s_scheme.rdx;
   unsigned long long m3v[3] = {0ull, 0ull, 0ull};
   const bool want_alpha = (NC == 3 || a.system >= 2) && (a.mode == 0) && (a.alpha_out != nullptr);
   if (tid < T && i0 + tid < nx) {
@@ -438,7 +432,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
 }
 
 template <int NC, int AI, bool P1, int PREC, int R = 3>
-__global__ void __launch_bounds__(kThreads1D) k_line1d(const StageArgs a) {
+__global__ void __launch_bounds__(kThreads1D) k_line1d(const __grid_constant__ StageArgs a) {
   extern __shared__ double sm[];
   line1d_tile<NC, AI, P1, PREC, kT1, R>(a, blockIdx.y, blockIdx.x,
                                         blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, sm);
@@ -446,7 +440,7 @@ __global__ void __launch_bounds__(kThreads1D) k_line1d(const StageArgs a) {
 
 // Latency layout of small 1D problems (lanes1d).
 template <int NC, int AI, bool P1, int PREC>
-__global__ void __launch_bounds__(kThreads1D) k_line1d_lanes(const StageArgs a) {
+__global__ void __launch_bounds__(kThreads1D) k_line1d_lanes(const __grid_constant__ StageArgs a) {
   extern __shared__ double sm[];
   constexpr int kL = lanes1d(NC, P1, PREC);
   line1d_tile<NC, AI, P1, PREC, cells_lanes1d(kL), 3, kL>(

@@ -18,6 +18,7 @@ namespace {
 // problem (blockIdx.y).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_alpha(const AlphaArgs a) {
+  pdl_start();
   const long long b = blockIdx.y;
   const long long plane = a.nx * a.ny;
   const double *Ub = a.U + b * a.nc * plane;
@@ -188,6 +189,7 @@ __device__ __forceinline__ StageArgs slot_stage_args(const SlotDev &S, int stage
 __global__ void __launch_bounds__(kEngineThreads, kEngineBlocksPerSM) k_engine(const EngineArgs e) {
   extern __shared__ double sm[];
   __shared__ int s_w;
+  pdl_start();
   const int cin = e.stage - 1, czero = (e.stage + 1) % 3;
   if (blockIdx.x == 0 && threadIdx.x == 0) e.counters[czero] = 0;
   const int ntiles = *e.ntiles, first = *e.first;
@@ -341,8 +343,7 @@ cudaError_t engine_prepare() {
 }
 
 cudaError_t launch_engine_stage(const EngineArgs &e, int grid, cudaStream_t s) {
-  k_engine<<<grid, kEngineThreads, engine_smem_bytes(), s>>>(e);
-  return cudaGetLastError();
+  return launch_chained(true, k_engine, dim3((unsigned)grid, 1, 1), kEngineThreads, engine_smem_bytes(), s, e);
 }
 
 cudaError_t launch_alpha(const AlphaArgs &a, cudaStream_t s) {

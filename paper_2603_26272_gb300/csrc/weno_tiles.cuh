@@ -512,9 +512,7 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
   // Phase 2: every x- and y-face of the tile once.  Lanes of a warp may mix
   // directions; the code path is the same (only the plane indices differ).
   const unsigned long long *al = a.alpha_in + b * 8;
-  const ReconParams rp4 = a.sp.rp[1], rp2 = a.sp.rp[0];
-  for (int f = tid; f < NFX + NFY; f += blockDim.x) {
-    int base, stride, dir, fr, fc;
+  auto locate = [&](int f, int &base, int &stride, int &dir, int &fr, int &fc) {
     if (f < NFX) {
       fr = f / (TX + 1);
       fc = f - fr * (TX + 1);
@@ -529,13 +527,29 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
       stride = W;
       dir = 1;
     }
-    const int pmn = 1 + dir, pmt = 2 - dir, pun = 4 + dir, put = 5 - dir;
+  };
+  auto face_state = [&](int base, int stride, int dir, int fr, int fc, FaceState &fs) {
+    const int pun = 4 + dir, put = 5 - dir;
     const int kL = base + (R - 1) * stride, kR = base + R * stride;
-    FaceState fs;
     if (!roe_face(pl[7 * REG + kL], pl[pun * REG + kL], pl[put * REG + kL], pl[6 * REG + kL],
                   pl[7 * REG + kR], pl[pun * REG + kR], pl[put * REG + kR], pl[6 * REG + kR],
                   gm1, fs))
-      record_status(a.status, 3, a.stage, b, j0 + (dir ? fr : fr), i0 + fc);
+      record_status(a.status, 3, a.stage, b, j0 + fr, i0 + fc);
+  };
+  auto store = [&](int dir, int fr, int fc, double F0, double F1, double F2, double F3) {
+    double *out = dir ? &fy[(fr * TX + fc) * 4] : &fx[(fr * (TX + 1) + fc) * 4];
+    out[0] = F0;
+    out[1 + dir] = F1;
+    out[2 - dir] = F2;
+    out[3] = F3;
+  };
+  const ReconParams rp4 = a.sp.rp[1], rp2 = a.sp.rp[0];
+  for (int f = tid; f < NFX + NFY; f += blockDim.x) {
+    int base, stride, dir, fr, fc;
+    locate(f, base, stride, dir, fr, fc);
+    const int pmn = 1 + dir, pmt = 2 - dir, pun = 4 + dir;
+    FaceState fs;
+    face_state(base, stride, dir, fr, fc, fs);
     const double A1 = field_speed(a, al + 4 * dir, 0, 4), A2 = field_speed(a, al + 4 * dir, 1, 4);
     const double A3 = field_speed(a, al + 4 * dir, 2, 4), A4 = field_speed(a, al + 4 * dir, 3, 4);
     double h1, h2, h3, h4;
@@ -565,11 +579,7 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
     }
     double F0, F1, F2, F3;
     backproject4(fs, h1, h2, h3, h4, F0, F1, F2, F3);
-    double *out = dir ? &fy[(fr * TX + fc) * 4] : &fx[(fr * (TX + 1) + fc) * 4];
-    out[0] = F0;
-    out[1 + dir] = F1;
-    out[2 - dir] = F2;
-    out[3] = F3;
+    store(dir, fr, fc, F0, F1, F2, F3);
   }
   __syncthreads();
 
@@ -899,12 +909,43 @@ __device__ __forceinline__ void euler2d_tile(const StageArgs &a, long long b, lo
     euler2d_tile_gen<TX, TY, AI, P1, PREC, R>(a, b, tile, zeroing_block, sm, tm);
 }
 
+// Programmatic dependent launch: a stage whose grid is small is bound by its
+// length, and 2 to 3 us of that are the launch itself.  Launched with the
+// attribute, the next stage's blocks are placed while this one runs (each block
+// lets them at its start) and wait, before they read anything, for it to have
+// ended with its memory visible; without the attribute both are no-ops.
+// Only for grids of at most one block per SM (and the engine's persistent
+// grid): blocks placed early beside running ones leave the SMs unevenly loaded
+// (20 x 1600 cells, 260 blocks: 79 -> 102 us a step), while 85 blocks gain
+// (shock-density N = 1600: 3.57 -> 2.92 ms for 73 steps) and 4 gain most
+// (advection N = 200: 2.93 -> 2.00 ms for 100 steps).
+__device__ __forceinline__ void pdl_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_chained(bool chain, void (*kern)(P...), dim3 grid, int threads, size_t smem,
+                           cudaStream_t s, const A &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // MINB: resident blocks per SM the register allocation must allow.
 // tm: tensor map of a.Uin (see euler2d_tile), used when a.use_tma is set.
 template <int TX, int TY, int NT, int MINB, int AI, bool P1, int PREC, int R = 3>
 __global__ void __launch_bounds__(NT, MINB)
     k_euler2d(const __grid_constant__ StageArgs a, const __grid_constant__ CUtensorMap tm) {
   extern __shared__ __align__(128) double sm[];
+  pdl_start();
   euler2d_tile<TX, TY, AI, P1, PREC, R>(a, blockIdx.z, blockIdx.x,
                                         blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, sm,
                                         a.use_tma ? &tm : nullptr);
@@ -924,6 +965,8 @@ inline int sm_count() {
   }
   return cached[dev];
 }
+
+inline bool one_per_sm(dim3 g) { return (long long)g.x * g.y * g.z <= sm_count(); }
 
 // Shared memory per SM the resident blocks of a launch may take (228 KB,
 // less 1 KB the hardware keeps per block).
@@ -947,8 +990,7 @@ cudaError_t launch_2d(const StageArgs &a_in, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long tiles = ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY);
   dim3 grid((unsigned)tiles, 1, (unsigned)a.nbatch);
-  kern<<<grid, NT, smem, s>>>(a, tm);
-  return cudaGetLastError();
+  return launch_chained(one_per_sm(grid), kern, grid, NT, smem, s, a, tm);
 }
 
 template <int AI, bool P1, int PREC, int R>
@@ -971,10 +1013,17 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     // Weights other than the default ones (without Ai, with a sensitivity term
     // that counts, p != 1) are built in three of the shapes (2, 8, 9; see
     // tile_shape_built), which keeps the library's build short.
-    // The other orders use 16x16 / 128 only, 3 blocks per SM at r = 2 and 2
-    // at r = 4, 5 (their wider stencils need more registers).
+    // The other orders use 16x15 / 128 only, 3 blocks per SM at r = 2 and 2
+    // at r = 4, 5 (their wider stencils need more registers): 511 faces, four a
+    // thread, where 16x16 had 544 and warp 0 a fifth round of them; a grid of no
+    // more such tiles than SMs, where a stage lasts as long as one thread's
+    // faces, in 8x8 / 160 (144 faces, one a thread).
     if constexpr (R != 3) {  // r = 2 fits the 168-register cap of 3 blocks per SM
-      return launch_2d<16, 16, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
+      if constexpr (P1) {
+        if (((a.nx + 15) / 16) * ((a.ny + 14) / 15) * a.nbatch <= sm_count())
+          return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
+      }
+      return launch_2d<16, 15, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
     } else if constexpr (!all_tile_shapes(AI, P1, PREC)) {
       switch (tile_shape_built(false, a.tile_variant)) {
         case 2: return launch_2d<16, 8, 64, 4, AI, P1, PREC>(a, s);
@@ -1007,20 +1056,20 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
       const int tl1 = a.nc == 3 ? cells_lanes1d(kL3) : cells_lanes1d(2);
       dim3 g2((unsigned)((a.nx + tl1 - 1) / tl1), (unsigned)a.nbatch, 1);
       if (a.nc == 3)
-        k_line1d_lanes<3, AI, P1, PREC>
-            <<<g2, kThreads1D, smem_line1d<3, cells_lanes1d(kL3), 3, kL3>(), s>>>(a);
+        return launch_chained(one_per_sm(g2), k_line1d_lanes<3, AI, P1, PREC>, g2, kThreads1D,
+                              smem_line1d<3, cells_lanes1d(kL3), 3, kL3>(), s, a);
       else if constexpr (PREC == 0)
-        k_line1d_lanes<1, AI, P1, PREC>
-            <<<g2, kThreads1D, smem_line1d<1, cells_lanes1d(2), 3, 2>(), s>>>(a);
-      return cudaGetLastError();
+        return launch_chained(one_per_sm(g2), k_line1d_lanes<1, AI, P1, PREC>, g2, kThreads1D,
+                              smem_line1d<1, cells_lanes1d(2), 3, 2>(), s, a);
     }
   }
   dim3 grid((unsigned)tiles, (unsigned)a.nbatch, 1);
   if (a.nc == 3)
-    k_line1d<3, AI, P1, PREC, R><<<grid, kThreads1D, smem_line1d<3, kT1, R>(), s>>>(a);
+    return launch_chained(one_per_sm(grid), k_line1d<3, AI, P1, PREC, R>, grid, kThreads1D, smem_line1d<3, kT1, R>(), s,
+                          a);
   else
-    k_line1d<1, AI, P1, PREC, R><<<grid, kThreads1D, smem_line1d<1, kT1, R>(), s>>>(a);
-  return cudaGetLastError();
+    return launch_chained(one_per_sm(grid), k_line1d<1, AI, P1, PREC, R>, grid, kThreads1D, smem_line1d<1, kT1, R>(), s,
+                          a);
 }
 
 }  // namespace

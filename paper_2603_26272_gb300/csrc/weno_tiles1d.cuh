@@ -434,6 +434,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
 template <int NC, int AI, bool P1, int PREC, int R = 3>
 __global__ void __launch_bounds__(kThreads1D) k_line1d(const __grid_constant__ StageArgs a) {
   extern __shared__ double sm[];
+  pdl_start();
   line1d_tile<NC, AI, P1, PREC, kT1, R>(a, blockIdx.y, blockIdx.x,
                                         blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, sm);
 }
@@ -442,6 +443,7 @@ __global__ void __launch_bounds__(kThreads1D) k_line1d(const __grid_constant__ S
 template <int NC, int AI, bool P1, int PREC>
 __global__ void __launch_bounds__(kThreads1D) k_line1d_lanes(const __grid_constant__ StageArgs a) {
   extern __shared__ double sm[];
+  pdl_start();
   constexpr int kL = lanes1d(NC, P1, PREC);
   line1d_tile<NC, AI, P1, PREC, cells_lanes1d(kL), 3, kL>(
       a, blockIdx.y, blockIdx.x, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, sm);

@@ -512,7 +512,9 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
   // Phase 2: every x- and y-face of the tile once.  Lanes of a warp may mix
   // directions; the code path is the same (only the plane indices differ).
   const unsigned long long *al = a.alpha_in + b * 8;
-  auto locate = [&](int f, int &base, int &stride, int &dir, int &fr, int &fc) {
+  const ReconParams rp4 = a.sp.rp[1], rp2 = a.sp.rp[0];
+  for (int f = tid; f < NFX + NFY; f += blockDim.x) {
+    int base, stride, dir, fr, fc;
     if (f < NFX) {
       fr = f / (TX + 1);
       fc = f - fr * (TX + 1);
@@ -527,29 +529,13 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
       stride = W;
       dir = 1;
     }
-  };
-  auto face_state = [&](int base, int stride, int dir, int fr, int fc, FaceState &fs) {
-    const int pun = 4 + dir, put = 5 - dir;
+    const int pmn = 1 + dir, pmt = 2 - dir, pun = 4 + dir, put = 5 - dir;
     const int kL = base + (R - 1) * stride, kR = base + R * stride;
+    FaceState fs;
     if (!roe_face(pl[7 * REG + kL], pl[pun * REG + kL], pl[put * REG + kL], pl[6 * REG + kL],
                   pl[7 * REG + kR], pl[pun * REG + kR], pl[put * REG + kR], pl[6 * REG + kR],
                   gm1, fs))
-      record_status(a.status, 3, a.stage, b, j0 + fr, i0 + fc);
-  };
-  auto store = [&](int dir, int fr, int fc, double F0, double F1, double F2, double F3) {
-    double *out = dir ? &fy[(fr * TX + fc) * 4] : &fx[(fr * (TX + 1) + fc) * 4];
-    out[0] = F0;
-    out[1 + dir] = F1;
-    out[2 - dir] = F2;
-    out[3] = F3;
-  };
-  const ReconParams rp4 = a.sp.rp[1], rp2 = a.sp.rp[0];
-  for (int f = tid; f < NFX + NFY; f += blockDim.x) {
-    int base, stride, dir, fr, fc;
-    locate(f, base, stride, dir, fr, fc);
-    const int pmn = 1 + dir, pmt = 2 - dir, pun = 4 + dir;
-    FaceState fs;
-    face_state(base, stride, dir, fr, fc, fs);
+      record_status(a.status, 3, a.stage, b, j0 + (dir ? fr : fr), i0 + fc);
     const double A1 = field_speed(a, al + 4 * dir, 0, 4), A2 = field_speed(a, al + 4 * dir, 1, 4);
     const double A3 = field_speed(a, al + 4 * dir, 2, 4), A4 = field_speed(a, al + 4 * dir, 3, 4);
     double h1, h2, h3, h4;
@@ -579,7 +565,11 @@ __device__ __forceinline__ void euler2d_tile_gen(const StageArgs &a, long long b
     }
     double F0, F1, F2, F3;
     backproject4(fs, h1, h2, h3, h4, F0, F1, F2, F3);
-    store(dir, fr, fc, F0, F1, F2, F3);
+    double *out = dir ? &fy[(fr * TX + fc) * 4] : &fx[(fr * (TX + 1) + fc) * 4];
+    out[0] = F0;
+    out[1 + dir] = F1;
+    out[2 - dir] = F2;
+    out[3] = F3;
   }
   __syncthreads();
 
@@ -1013,17 +1003,10 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     // Weights other than the default ones (without Ai, with a sensitivity term
     // that counts, p != 1) are built in three of the shapes (2, 8, 9; see
     // tile_shape_built), which keeps the library's build short.
-    // The other orders use 16x15 / 128 only, 3 blocks per SM at r = 2 and 2
-    // at r = 4, 5 (their wider stencils need more registers): 511 faces, four a
-    // thread, where 16x16 had 544 and warp 0 a fifth round of them; a grid of no
-    // more such tiles than SMs, where a stage lasts as long as one thread's
-    // faces, in 8x8 / 160 (144 faces, one a thread).
+    // The other orders use 16x16 / 128 only, 3 blocks per SM at r = 2 and 2
+    // at r = 4, 5 (their wider stencils need more registers).
     if constexpr (R != 3) {  // r = 2 fits the 168-register cap of 3 blocks per SM
-      if constexpr (P1) {
-        if (((a.nx + 15) / 16) * ((a.ny + 14) / 15) * a.nbatch <= sm_count())
-          return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
-      }
-      return launch_2d<16, 15, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
+      return launch_2d<16, 16, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
     } else if constexpr (!all_tile_shapes(AI, P1, PREC)) {
       switch (tile_shape_built(false, a.tile_variant)) {
         case 2: return launch_2d<16, 8, 64, 4, AI, P1, PREC>(a, s);
@@ -1065,11 +1048,11 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
   }
   dim3 grid((unsigned)tiles, (unsigned)a.nbatch, 1);
   if (a.nc == 3)
-    return launch_chained(one_per_sm(grid), k_line1d<3, AI, P1, PREC, R>, grid, kThreads1D, smem_line1d<3, kT1, R>(), s,
-                          a);
+    return launch_chained(one_per_sm(grid), k_line1d<3, AI, P1, PREC, R>, grid, kThreads1D,
+                          smem_line1d<3, kT1, R>(), s, a);
   else
-    return launch_chained(one_per_sm(grid), k_line1d<1, AI, P1, PREC, R>, grid, kThreads1D, smem_line1d<1, kT1, R>(), s,
-                          a);
+    return launch_chained(one_per_sm(grid), k_line1d<1, AI, P1, PREC, R>, grid, kThreads1D,
+                          smem_line1d<1, kT1, R>(), s, a);
 }
 
 }  // namespace

@@ -1003,10 +1003,22 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     // Weights other than the default ones (without Ai, with a sensitivity term
     // that counts, p != 1) are built in three of the shapes (2, 8, 9; see
     // tile_shape_built), which keeps the library's build short.
-    // The other orders use 16x16 / 128 only, 3 blocks per SM at r = 2 and 2
-    // at r = 4, 5 (their wider stencils need more registers).
+    // The other orders use 16x15 / 128, 3 blocks per SM at r = 2 and 2 at
+    // r = 4, 5 (their wider stencils need more registers): 511 faces, four a
+    // thread, where 16x16 has 544 and every block's warp 0 a fifth round of them
+    // on the same sub-partition (300^2 steps of orders 4 / 8 / 10: 830 / 2112 /
+    // 3027 -> 755 / 1826 / 2605 us; 1024 x 512, orders 8 / 10: 9.10 / 13.07 ->
+    // 8.72 / 12.50 ms).  A grid of no more such tiles than SMs, where a stage
+    // lasts as long as one thread's faces, takes 8x8 / 160 (144 faces, one a
+    // thread): 64^2, orders 8 / 10: 812 / 1158 -> 230 / 314 us; 150^2 (100 of the
+    // large tiles): 811 / 1159 -> 657 / 909 us.  Above that line the halo costs
+    // more than the length gives.
     if constexpr (R != 3) {  // r = 2 fits the 168-register cap of 3 blocks per SM
-      return launch_2d<16, 16, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
+      if constexpr (P1) {
+        if (((a.nx + 15) / 16) * ((a.ny + 14) / 15) * a.nbatch <= sm_count())
+          return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
+      }
+      return launch_2d<16, 15, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
     } else if constexpr (!all_tile_shapes(AI, P1, PREC)) {
       switch (tile_shape_built(false, a.tile_variant)) {
         case 2: return launch_2d<16, 8, 64, 4, AI, P1, PREC>(a, s);

@@ -904,11 +904,14 @@ __device__ __forceinline__ void euler2d_tile(const StageArgs &a, long long b, lo
 // attribute, the next stage's blocks are placed while this one runs (each block
 // lets them at its start) and wait, before they read anything, for it to have
 // ended with its memory visible; without the attribute both are no-ops.
-// Only for grids of at most one block per SM (and the engine's persistent
-// grid): blocks placed early beside running ones leave the SMs unevenly loaded
-// (20 x 1600 cells, 260 blocks: 79 -> 102 us a step), while 85 blocks gain
-// (shock-density N = 1600: 3.57 -> 2.92 ms for 73 steps) and 4 gain most
-// (advection N = 200: 2.93 -> 2.00 ms for 100 steps).
+// Only where the blocks of two stages fit on SMs of their own: a block placed
+// early beside a running one shares its SM while others are idle (order 8 of
+// 14,000 cells, 111 blocks: 158 us a step plain, 286 chained; FP32 of 96^2, 144
+// blocks: 98 and 114; order 6 of 96^2: 123.5 and 144.5).  The lane layout, bound
+// by latency and not by the FP64 pipe, gains up to one block per SM (85 blocks,
+// shock-density N = 1600: 3.57 -> 2.92 ms for 73 steps; 4 blocks, advection
+// N = 200: 2.93 -> 2.00 ms for 100 steps), and so does the engine's persistent
+// grid; 20 x 1600 cells, 260 blocks: 79 -> 102 us.
 __device__ __forceinline__ void pdl_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -956,7 +959,10 @@ inline int sm_count() {
   return cached[dev];
 }
 
-inline bool one_per_sm(dim3 g) { return (long long)g.x * g.y * g.z <= sm_count(); }
+// Whether the blocks of `times` such grids find an SM each.
+inline bool fits(dim3 g, int times = 1) {
+  return times * (long long)g.x * g.y * g.z <= sm_count();
+}
 
 // Shared memory per SM the resident blocks of a launch may take (228 KB,
 // less 1 KB the hardware keeps per block).
@@ -980,7 +986,7 @@ cudaError_t launch_2d(const StageArgs &a_in, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long tiles = ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY);
   dim3 grid((unsigned)tiles, 1, (unsigned)a.nbatch);
-  return launch_chained(one_per_sm(grid), kern, grid, NT, smem, s, a, tm);
+  return launch_chained(fits(grid, 2), kern, grid, NT, smem, s, a, tm);
 }
 
 template <int AI, bool P1, int PREC, int R>
@@ -1051,19 +1057,19 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
       const int tl1 = a.nc == 3 ? cells_lanes1d(kL3) : cells_lanes1d(2);
       dim3 g2((unsigned)((a.nx + tl1 - 1) / tl1), (unsigned)a.nbatch, 1);
       if (a.nc == 3)
-        return launch_chained(one_per_sm(g2), k_line1d_lanes<3, AI, P1, PREC>, g2, kThreads1D,
+        return launch_chained(fits(g2), k_line1d_lanes<3, AI, P1, PREC>, g2, kThreads1D,
                               smem_line1d<3, cells_lanes1d(kL3), 3, kL3>(), s, a);
       else if constexpr (PREC == 0)
-        return launch_chained(one_per_sm(g2), k_line1d_lanes<1, AI, P1, PREC>, g2, kThreads1D,
+        return launch_chained(fits(g2), k_line1d_lanes<1, AI, P1, PREC>, g2, kThreads1D,
                               smem_line1d<1, cells_lanes1d(2), 3, 2>(), s, a);
     }
   }
   dim3 grid((unsigned)tiles, (unsigned)a.nbatch, 1);
   if (a.nc == 3)
-    return launch_chained(one_per_sm(grid), k_line1d<3, AI, P1, PREC, R>, grid, kThreads1D,
+    return launch_chained(fits(grid, 2), k_line1d<3, AI, P1, PREC, R>, grid, kThreads1D,
                           smem_line1d<3, kT1, R>(), s, a);
   else
-    return launch_chained(one_per_sm(grid), k_line1d<1, AI, P1, PREC, R>, grid, kThreads1D,
+    return launch_chained(fits(grid, 2), k_line1d<1, AI, P1, PREC, R>, grid, kThreads1D,
                           smem_line1d<1, kT1, R>(), s, a);
 }
 

@@ -989,6 +989,19 @@ cudaError_t launch_2d(const StageArgs &a_in, cudaStream_t s) {
   return launch_chained(fits(grid, 2), kern, grid, NT, smem, s, a, tm);
 }
 
+template <int TX, int TY>
+inline long long tiles_2d(const StageArgs &a) {
+  return ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY) * a.nbatch;
+}
+
+// What a stage of `tiles` tiles costs that give every thread `faces` faces, in
+// tenths of a face of a full wave: a face takes 127 us (r = 5) where per_sm
+// blocks share an SM and 77 where one has it alone.
+inline long long wave_cost(long long tiles, int faces, int per_sm) {
+  const long long wave = (long long)sm_count() * per_sm, rest = tiles % wave;
+  return faces * (10 * (tiles / wave) + (rest == 0 ? 0 : rest <= sm_count() ? 6 : 10));
+}
+
 template <int AI, bool P1, int PREC, int R>
 cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
   if (a.ndim == 2) {
@@ -1019,12 +1032,18 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     // thread): 64^2, orders 8 / 10: 812 / 1158 -> 230 / 314 us; 150^2 (100 of the
     // large tiles): 811 / 1159 -> 657 / 909 us.  Above that line the halo costs
     // more than the length gives.
+    // Between them, the shape whose last wave is fuller: 20x15 / 128 (635 faces,
+    // five a thread) where wave_cost says so (orders 8 / 10, 16x15 -> 20x15:
+    // 220x190 1193 / 1694 -> 834 / 1182 us, 300^2 1826 / 2605 -> 1493 / 2120,
+    // 512^2 4659 / 6657 -> 4378 / 6253).
     if constexpr (R != 3) {  // r = 2 fits the 168-register cap of 3 blocks per SM
+      constexpr int kPerSM = R == 2 ? 3 : 2;
       if constexpr (P1) {
-        if (((a.nx + 15) / 16) * ((a.ny + 14) / 15) * a.nbatch <= sm_count())
-          return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
+        if (tiles_2d<16, 15>(a) <= sm_count()) return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
+        if (wave_cost(tiles_2d<20, 15>(a), 5, kPerSM) < wave_cost(tiles_2d<16, 15>(a), 4, kPerSM))
+          return launch_2d<20, 15, 128, kPerSM, AI, P1, PREC, R>(a, s);
       }
-      return launch_2d<16, 15, 128, (R == 2 ? 3 : 2), AI, P1, PREC, R>(a, s);
+      return launch_2d<16, 15, 128, kPerSM, AI, P1, PREC, R>(a, s);
     } else if constexpr (!all_tile_shapes(AI, P1, PREC)) {
       switch (tile_shape_built(false, a.tile_variant)) {
         case 2: return launch_2d<16, 8, 64, 4, AI, P1, PREC>(a, s);

@@ -1,7 +1,8 @@
-"""GPU: the tile the other orders take on grids with no more 16x16 tiles than the
-GPU has SMs, against the one of larger grids: a problem alone takes the small tile,
-the same problem repeated in a batch the large one, and every face is the same
-arithmetic, so the right-hand sides are equal bit for bit.
+"""GPU: the tile the other orders take on grids with few tiles, against those of
+larger grids: a problem alone takes the 8x8 tile, the same problem repeated in a
+batch one of the large ones (16x15 for the first three sizes, 20x15 for the last
+two), and every face is the same arithmetic, so the right-hand sides are equal
+bit for bit.
 """
 import numpy as np
 import pytest
@@ -22,7 +23,7 @@ def _cuda():
 @pytest.mark.parametrize("bc", ["transmissive", "periodic"])
 @pytest.mark.parametrize("nx,ny", [(1, 1), (7, 9), (8, 8), (17, 16), (50, 33)])
 @pytest.mark.parametrize("order", [4, 8, 10])
-def test_small_tile_bitwise_large_tile(order, nx, ny, bc):
+def test_small_tile_bitwise_large_tiles(order, nx, ny, bc):
     U = wl.random_smooth_2d(nx=64, ny=64, seed=8)["U"][:, :, :ny, :nx].copy()
     U[:, :, ny // 2:, nx // 2:] *= 1.7
     tiles = -(-nx // 16) * -(-ny // 16)

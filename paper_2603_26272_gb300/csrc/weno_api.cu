@@ -290,8 +290,10 @@ weno_status read_status(const Ctx &c) {
 // Tile autotuner for the 2D stage kernel.  The first call on a new problem
 // shape times every tile variant on the caller's data (one right-hand-side
 // stage each, written into the scratch state U1) and caches the fastest; all
-// variants compute bitwise the same result.  WENO_TILE2D=0|1|2 in the
-// environment forces a variant and skips the timing.
+// variants compute bitwise the same result.  WENO_TILE2D=0..10 in the
+// environment forces a variant and skips the timing.  Weights other than the
+// default ones have three shapes built; the other numbers stand for one of them
+// (tile_shape_built).
 // ---------------------------------------------------------------------------
 std::mutex g_tune_mu;
 std::map<std::tuple<long long, long long, long long, int, int, int>, int> g_tune;

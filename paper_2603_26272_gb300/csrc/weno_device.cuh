@@ -1033,7 +1033,9 @@ __device__ __forceinline__ bool face_exponents(int a, Diff diff, int (&E)[NC], i
 // differences w of the states and g of the fluxes in units of 2^k0, and the
 // speed A; k is the scale of the result, or INT_MIN where the field is left
 // to FP64.  Calls, so that their code is there once: inlined for every field,
-// a face's code outgrows the instruction cache.
+// a face's code outgrows the instruction cache (2048^2 step: 15.8 ms inlined
+// with 5.0 no-instruction stalls per issue, 9.14 ms as calls with the x- and
+// y-faces in one loop).
 struct FieldSum {
   fx::i64 S;
   int k;

@@ -12,8 +12,16 @@
 // of 2^-57 of the largest difference, in every difference, is below the
 // rounding FP64 gives it (2^-53 per operation).
 //
-// Number formats (tests/test_kernel_fixed.py restates them and measures the
-// error against quadruple precision):
+// Measured at 2048^2, FP64, one step: 33.5 ms with the reconstruction and the
+// projections on the FP64 pipe, 16.0 ms with the reconstruction here, 9.16 ms
+// with the projections (project) and the smooth stencils (smooth_term) too,
+// 7.85 ms with the scheme's constants from the host and the speed maxima
+// filtered in FP32.  What is left is bound by both: FP64 pipe 57 %, integer
+// (alu) 36 %, 44 % of the issue slots (1024^2, 11.3k instructions and 214 FP64
+// operations per cell and stage).
+//
+// Number formats (tests/test_kernel_fixed.py compiles this header for the host
+// and measures the error against quadruple precision):
 //  * differences and what is linear in them (second differences, candidate
 //    fluxes, the fifth difference): 64-bit integers in units of 2^-57 of the
 //    power of two above the largest of the ten differences of a field -- exact
@@ -456,7 +464,9 @@ WENO_FX float rcpf(float x) {
 // differences, with an error below 2^-21 of max G max |r_k - rm|, it is good
 // to 2 units (2^-58 of the bound on the projected differences) where that
 // product is at most 2^22 units, from about 70 cells a wavelength on.
-// |d_j| < 2^61: a field's differences over 4.  Returns whether it is, and the term in units.
+// |d_j| < 2^61: a field's differences over 4.  Returns whether it is, and the
+// term in units.  (About 80 FP32 operations a flux, where the weights take
+// several hundred integer ones.)
 // SENS: a sensitivity term would lower G, so the term then has to vanish (at
 // most half a unit); without it (epsilon <= 2^-126) the same holds unless
 // every b_k is above 2^18 units squared, 2^25 times what it could be.
@@ -531,9 +541,6 @@ WENO_FX double from_fixed(i64 S, int k) {
   const u64 b = r + ((u64)(i64)(1085 + k - n) << 52);
   return bitsd(S == 0 ? 0 : (S < 0 ? b | 0x8000000000000000ull : b));
 }
-
-// 2^k / 6 for -1019 <= k <= 1026.
-WENO_FX double sixth(int k) { return bitsd(dbits(1.0 / 6.0) + ((u64)(i64)k << 52)); }
 
 }  // namespace fx
 }  // namespace weno

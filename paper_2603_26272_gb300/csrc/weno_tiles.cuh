@@ -1039,7 +1039,8 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     if constexpr (R != 3) {  // r = 2 fits the 168-register cap of 3 blocks per SM
       constexpr int kPerSM = R == 2 ? 3 : 2;
       if constexpr (P1) {
-        if (tiles_2d<16, 15>(a) <= sm_count()) return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
+        if (tiles_2d<16, 15>(a) <= sm_count())
+          return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
         if (wave_cost(tiles_2d<20, 15>(a), 5, kPerSM) < wave_cost(tiles_2d<16, 15>(a), 4, kPerSM))
           return launch_2d<20, 15, 128, kPerSM, AI, P1, PREC, R>(a, s);
       }

@@ -460,10 +460,12 @@ WENO_FX float rcpf(float x) {
 //   c = rm + sum_k D_k G_k (r_k - rm) / (20 + sum_k D_k G_k), G_k = T / b_k,
 // the second term is far below a unit, or a few units, wherever the stencil
 // resolves its data (G is the eighth power of the phase per cell, r_k - rm its
-// third).  Computed in FP32 on the exact second differences and their exact
-// differences, with an error below 2^-21 of max G max |r_k - rm|, it is good
-// to 2 units (2^-58 of the bound on the projected differences) where that
-// product is at most 2^22 units, from about 70 cells a wavelength on.
+// third).  Computed in FP32 on the exact second differences, their exact
+// differences and the exact fifth one, so that nothing cancels but in forming
+// r_k - rm, whose largest is at least half the largest of its terms: the error
+// is below 2^-21 of max G max |r_k - rm|, which is 2 units (2^-58 of the bound
+// on the projected differences) where that product is at most 2^22 units, from
+// about 70 cells a wavelength on.
 // |d_j| < 2^61: a field's differences over 4.  Returns whether it is, and the
 // term in units.  (About 80 FP32 operations a flux, where the weights take
 // several hundred integer ones.)
@@ -475,7 +477,12 @@ WENO_FX bool smooth_term(const i64 (&d)[5], int &corr) {
   const i64 s0 = d[1] - d[0], s1 = d[2] - d[1], s2 = d[3] - d[2], s3 = d[4] - d[3];
   const float a0 = to_float(s0), a1 = to_float(s1), a2 = to_float(s2), a3 = to_float(s3);
   const float f1 = to_float(d[1]), f2 = to_float(d[2]), f3 = to_float(d[3]);
-  const float e2 = to_float(s1 - s2), r5 = ffma(3.0f, e2, to_float(s3 - s0));
+  const i64 q = s1 - s2, l = s3 - s0;
+  const float e2 = to_float(q), f5 = ffma(3.0f, e2, to_float(l));
+  // l + 3 q is the fifth difference.  It can cancel to far below both, so where
+  // it fits 64 bits it is formed in them: FP32's 2^-24 of q would be noise in
+  // T, 1e6 units in the term of a cubic.
+  const float r5 = fabsf(f5) < 0x1p30f ? to_float((i64)((u64)l + 3 * (u64)q)) : f5;
   const float t0 = ffma(2.0f, f1, a0), t1 = fadd(f1, f2), t2 = ffma(2.0f, f2, -a2),
               t3 = ffma(3.0f, a3, fmul(-2.0f, f3));
   const float b0 = ffma(fmul(13.0f, a0), a0, fmul(fmul(3.0f, t0), t0));

@@ -1010,11 +1010,12 @@ __device__ __forceinline__ void backproject3(const FaceState &f, double h1, doub
 }
 
 // Exponent codes of a face's five pairs (weno_fixed.cuh) with fluxes aligned
-// to 2^a times the states, top the largest of the codes: false if a difference
-// is outside the packed range.
+// to 2^a (components 0 and 2 to 2^a1 too) times the states, top the largest of
+// the codes: false if a difference is outside the packed range.
 template <int NC, class Diff>
-__device__ __forceinline__ bool face_exponents(int a, Diff diff, int (&E)[NC], int &top) {
-  top = 0;
+__device__ __forceinline__ bool face_exponents(int a, int a1, Diff diff, int (&E)[NC], int &B0,
+                                               int &B2, int &top) {
+  top = B2 = 0;
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
     int eu = 0, ef = 0;
@@ -1024,7 +1025,9 @@ __device__ __forceinline__ bool face_exponents(int a, Diff diff, int (&E)[NC], i
       ef = max(ef, fx::packed_exponent(diff(1, q, j)));
     }
     top = max(top, max(eu, ef));
-    E[q] = max(eu, ef - a);
+    E[q] = fx::aligned(eu, ef, a);
+    if (q == 0) B0 = fx::aligned(eu, ef, a1);
+    if (NC == 4 && q == 2) B2 = fx::aligned(eu, ef, a1);
   }
   return top < fx::kWide;
 }
@@ -1156,47 +1159,49 @@ __device__ __forceinline__ double field_lanes(const fx::i64 (&v)[5], const fx::L
 }
 
 // 6 h of the fields of one face from its packed differences diff(s, q, j) of the
-// state (s = 0) and the physical flux (s = 1), component q, pair j; KA[m] and a: the fields'
-// speeds (fx::speed).
+// state (s = 0) and the physical flux (s = 1), component q, pair j; KA[m]: the fields' speeds
+// (fx::speed) with the exponents a (acoustic fields) and a1 (the others).
 template <int NC, int AI, class Diff, class Wide, class RP>
-__device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb *KA, int a,
+__device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb *KA, int a, int a1,
                                             Diff diff, RP rp, Wide wide, double (&h)[NC]) {
-  int E[NC], top;
-  bool ok = face_exponents<NC>(a, diff, E, top);
+  int E[NC], B0, B2, top;
+  bool ok = face_exponents<NC>(a, a1, diff, E, B0, B2, top);
   if (top == 0) {  // nothing varies over the stencil
 #pragma unroll
     for (int m = 0; m < NC; ++m) h[m] = 0.0;
     return;
   }
   const fx::LeftRows<NC> rows =
-      fx::left_rows<NC>(E, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic), __dmul_rn(fs.b1, fs.un),
-                        __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
+      fx::left_rows<NC>(E, B0, B2, a, a1, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic),
+                        __dmul_rn(fs.b1, fs.un), __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
   ok = ok && rows.emax < 2047;
   fx::i64 w[5], g[5];
   auto field = [&](int m, int k) {
     const FieldValue f = field_call<AI>(w[0], w[1], w[2], w[3], w[4], g[0], g[1], g[2], g[3], g[4],
-                                        KA[m], k + a - 1592, rp(m));
+                                        KA[m], k - 1592, rp(m));
     h[m] = ok && !f.wide ? f.h6 : 6.0 * wide(m);
   };
   if constexpr (NC == 4) {
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
-      w[j] = fx::project_shear(rows, E, 0, diff(0, 0, j), diff(0, 2, j));
-      g[j] = fx::project_shear(rows, E, a, diff(1, 0, j), diff(1, 2, j));
+      w[j] = fx::project_shear(rows, B0, 0, diff(0, 0, j), diff(0, 2, j));
+      g[j] = fx::project_shear(rows, B0, a1, diff(1, 0, j), diff(1, 2, j));
     }
-    field(2, rows.us);
+    field(2, rows.us + a1);
   }
   // the states, then the physical fluxes (a loop: half the code to fetch)
   fx::Proj U[5], F[5] = {};
 #pragma unroll 1
   for (int s = 0; s < 2; ++s) {
+    const int as = s ? a : 0, as1 = s ? a1 : 0;
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
       U[j] = F[j];
       fx::u64 v[NC];
 #pragma unroll
       for (int q = 0; q < NC; ++q) v[q] = diff(s, q, j);
-      F[j] = fx::project<NC>(rows, E, s ? a : 0, v);
+      F[j] = fx::project<NC>(rows, E, as, as1, v);
+      F[j].r = fx::entropy<NC>(rows, as, as1, F[j]);
     }
   }
   auto part = [&](auto of) {
@@ -1206,12 +1211,12 @@ __device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb 
       g[j] = of(F[j]);
     }
   };
-  part([](const fx::Proj &p) { return p.r - p.z; });
-  field(1, rows.um);
+  part([](const fx::Proj &p) { return p.r; });
+  field(1, rows.ue + a1);
   part([](const fx::Proj &p) { return p.z + p.tc; });
-  field(0, rows.um);
+  field(0, rows.um + a);
   part([](const fx::Proj &p) { return p.z - p.tc; });
-  field(NC - 1, rows.um);
+  field(NC - 1, rows.um + a);
 }
 
 }  // namespace weno

@@ -279,18 +279,17 @@ WENO_FX u64 pack(double x) {
   return zero ? 0 : ((((i64)b < 0 ? 0 - m : m) << 10) | (u64)(in ? e - 511 : kWide));
 }
 WENO_FX int packed_exponent(u64 w) { return (int)(w & 0x3FF); }
-// Sign-extending shift of the packed mantissa; a count of 64 or more leaves
-// the sign.
-WENO_FX i64 packed_value(u64 w, int n) {
-  const i64 v = (i64)(w & ~0x3FFull);
+// Shift right with the sign; a count of 64 or more (or below 0) leaves the sign.
+WENO_FX i64 shr_signed(i64 v, int n) {
 #ifdef __CUDA_ARCH__
   i64 r;
   asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
   return r;
 #else
-  return v >> (n > 63 ? 63 : n);
+  return v >> ((unsigned)n > 63u ? 63 : n);
 #endif
 }
+WENO_FX i64 packed_value(u64 w, int n) { return shr_signed((i64)(w & ~0x3FFull), n); }
 
 // A number as two limbs, 2^32 h + 2 l (its lowest bit dropped): all products
 // of limbs are signed 32 x 32 -> 64 bits.
@@ -340,32 +339,43 @@ WENO_FX i64 times_speed(const Limb &A, i64 w) {
   return over63(v);
 }
 
+// Exponent code of a component: the largest of its states' and its fluxes' over 2^a.
+WENO_FX int aligned(int eu, int ef, int a) { return imax(eu, ef ? ef - a : 0); }
+
 // The left eigenvectors of a face in the form project4 (NC = 4) and project3
 // (NC = 3) apply them: with z = b2 r - t2 m_n - t3 m_t + b1 E and
 // tc = t1 r - ic m_n the fields are z + tc, r - z, (m_t - ut r,) z - tc.
-// um: the scale of z, tc and r, projected values are x 2^(1592 - um), a field
-// below 2^61.6; us: that of m_t - ut r.  emax: the largest exponent among the
-// coefficients (2047: not finite).
+// Three scales, each that of the terms its sums are made of, so that no field
+// is cut where FP64 would keep it: um of z and tc (r is no term of theirs:
+// beside a dense cell its scale would be far above them), ue of the entropy
+// field r - z, us of the shear field.  A projected state is x 2^(1592 - u), a
+// field below 2^61.6; fluxes are 2^a (z and tc) and 2^a1 (the two fields that
+// move with the flow, whose speed may be far below the sound speed) times as
+// large.  E: the components' exponents with 2^a, B0 and B2 of components 0 and
+// 2 with 2^a1.  emax: the largest exponent among the coefficients (2047: not
+// finite).
 template <int NC>
 struct LeftRows {
   Limb zr, zn, zt, zE, tr, tn, sr;
-  int um, us, emax;
+  int um, ue, us, emax;
 };
 template <int NC>
-WENO_FX LeftRows<NC> left_rows(const int (&E)[NC], double b2, double b1, double t1, double t2,
-                               double t3, double ic, double ut) {
+WENO_FX LeftRows<NC> left_rows(const int (&E)[NC], int B0, int B2, int a, int a1, double b2,
+                               double b1, double t1, double t2, double t3, double ic, double ut,
+                               int least = 0) {
   LeftRows<NC> o;
   const int e1 = exponent(b1), e2 = exponent(b2), f1 = exponent(t1), f2 = exponent(t2),
             f3 = exponent(t3), fc = exponent(ic), fu = exponent(ut);
   o.emax = imax(imax(imax(e1, e2), imax(f1, f2)), imax(fc, NC == 4 ? imax(f3, fu) : 0));
-  o.um = imax(imax(imax(e2, f1), 1023) + E[0], imax(imax(f2, fc) + E[1], e1 + E[NC - 1]));
+  o.um = imax(imax(imax(e2, f1) + E[0], least), imax(imax(f2, fc) + E[1], e1 + E[NC - 1]));
   o.us = 0;
   if (NC == 4) {
     o.um = imax(o.um, f3 + E[2]);
-    o.us = imax(fu + E[0], 1023 + E[2]);
+    o.us = imax(fu + B0, 1023 + B2);
     o.zt = coefficient(-t3, E[2], o.um);
-    o.sr = coefficient(-ut, E[0], o.us);
+    o.sr = coefficient(-ut, B0, o.us);
   }
+  o.ue = imax(o.um + a - a1, 1023 + B0);
   o.zr = coefficient(b2, E[0], o.um);
   o.zn = coefficient(-t2, E[1], o.um);
   o.zE = coefficient(b1, E[NC - 1], o.um);
@@ -373,14 +383,15 @@ WENO_FX LeftRows<NC> left_rows(const int (&E)[NC], double b2, double b1, double 
   o.tn = coefficient(-ic, E[1], o.um);
   return o;
 }
-// A difference vector's projections from its packed components v[q], with
-// a = 0 for states, the speeds' exponent for physical fluxes: z, tc and r, and
-// apart (it lives no longer than its own field) s = m_t - ut r.
+// A difference vector's projections from its packed components v[q], and apart
+// (it lives no longer than its own field) s = m_t - ut r; a = a1 = 0 for
+// states, the speeds' exponents for physical fluxes.  r is in units of the
+// entropy field (entropy).
 struct Proj {
   i64 z, tc, r;
 };
 template <int NC>
-WENO_FX Proj project(const LeftRows<NC> &c, const int (&E)[NC], int a, const u64 (&v)[NC]) {
+WENO_FX Proj project(const LeftRows<NC> &c, const int (&E)[NC], int a, int a1, const u64 (&v)[NC]) {
   Limb d[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) d[q] = limb(packed_value(v[q], E[q] + a + 2 - packed_exponent(v[q])));
@@ -391,13 +402,32 @@ WENO_FX Proj project(const LeftRows<NC> &c, const int (&E)[NC], int a, const u64
   mac(z, c.zE, d[NC - 1]);
   mac(t, c.tr, d[0]);
   mac(t, c.tn, d[1]);
-  return Proj{over63(z), over63(t), packed_value(v[0], c.um + a - 1018 - packed_exponent(v[0]))};
+  return Proj{over63(z), over63(t), packed_value(v[0], c.ue + a1 - 1018 - packed_exponent(v[0]))};
+}
+template <int NC>
+WENO_FX i64 entropy(const LeftRows<NC> &c, int a, int a1, const Proj &p) {
+  return p.r - shr_signed(p.z, c.ue + a1 - c.um - a);
+}
+WENO_FX i64 project_shear(const LeftRows<4> &c, int B0, int a1, u64 rho, u64 mt) {
+  Acc u = {0, 0};
+  mac(u, c.sr, limb(packed_value(rho, B0 + a1 + 2 - packed_exponent(rho))));
+  return over63(u) + packed_value(mt, c.us + a1 - 1018 - packed_exponent(mt));
+}
+#ifndef __CUDACC__
+// One speed exponent and one scale for all fields (host tests).
+template <int NC>
+WENO_FX LeftRows<NC> left_rows(const int (&E)[NC], double b2, double b1, double t1, double t2,
+                               double t3, double ic, double ut) {
+  return left_rows<NC>(E, E[0], E[2], 0, 0, b2, b1, t1, t2, t3, ic, ut, 1023 + E[0]);
+}
+template <int NC>
+WENO_FX Proj project(const LeftRows<NC> &c, const int (&E)[NC], int a, const u64 (&v)[NC]) {
+  return project<NC>(c, E, a, a, v);
 }
 WENO_FX i64 project_shear(const LeftRows<4> &c, const int (&E)[4], int a, u64 rho, u64 mt) {
-  Acc u = {0, 0};
-  mac(u, c.sr, limb(packed_value(rho, E[0] + a + 2 - packed_exponent(rho))));
-  return over63(u) + packed_value(mt, c.us + a - 1018 - packed_exponent(mt));
+  return project_shear(c, E[0], a, rho, mt);
 }
+#endif
 
 // The stencil differences g + x of f^+ become those of the mirrored f^-:
 // x - g in reverse order.

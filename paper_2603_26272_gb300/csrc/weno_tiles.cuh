@@ -609,10 +609,12 @@ __device__ __forceinline__ void normal_flux(double rho, double mn, double mt, do
 }
 
 // The GLF speeds of a problem in fixed point, per direction (fx::speed), and
-// the exponents above them; the block's first threads form them once.
+// the exponents above them, ea of the acoustic fields and eb of those that move
+// with the flow (u = 0 gives the latter none: 2^-300 of the former stands for
+// it); the block's first threads form them once.
 struct Speeds {
   fx::Limb ka[2][4];
-  int ea[2];
+  int ea[2], eb[2];
 };
 __device__ __forceinline__ void make_speeds(const StageArgs &a, long long b, int nc, Speeds &s) {
   const int dir = threadIdx.x >> 2, m = threadIdx.x & 3;
@@ -621,8 +623,12 @@ __device__ __forceinline__ void make_speeds(const StageArgs &a, long long b, int
   unsigned long long top = al[0];
   for (int q = 1; q < nc; ++q) top = max(top, al[q]);
   const int ea = fx::exponent(bits2d(top)) - 1022;
-  s.ka[dir][m] = fx::speed(field_speed(a, al, m, nc), ea);
-  if (m == 0) s.ea[dir] = ea;
+  const int eb = max(fx::exponent(field_speed(a, al, 1, nc)) - 1022, ea - 300);
+  s.ka[dir][m] = fx::speed(field_speed(a, al, m, nc), m == 0 || m == nc - 1 ? ea : eb);
+  if (m == 0) {
+    s.ea[dir] = ea;
+    s.eb[dir] = eb;
+  }
 }
 
 // Field m of face (fr, fc) along DIR in FP64 from the staged cells (less its
@@ -739,7 +745,7 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long lo
     if constexpr (kPacked) {
       const fx::u64 *const pf = dp + p0;
       face_fields<4, AI>(
-          fs, sp.ka[dir], sp.ea[dir],
+          fs, sp.ka[dir], sp.ea[dir], sp.eb[dir],
           [&](int s, int q, int j) { return pf[(s ? (q == 0 ? 1 : 3 + q) : q) * ND + j * ps]; },
           [&](int m) -> const ReconParams & { return (m == 0 || m == 3) ? rp4 : rp2; },
           [&](int m) {

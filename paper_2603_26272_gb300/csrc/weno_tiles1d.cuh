@@ -204,24 +204,25 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     auto diff = [&](int s, int c, int j) {
       return dp[(s ? (c == 0 ? 1 : 2 + c) : c) * ND + f + j];
     };
-    int E[3], top;
-    const int ea = s_sp.ea[0];
-    bool ok = face_exponents<3>(ea, diff, E, top);
+    int E[3], B0, B2, top;
+    const int ea = s_sp.ea[0], eb = s_sp.eb[0];
+    bool ok = face_exponents<3>(ea, eb, diff, E, B0, B2, top);
     const fx::LeftRows<3> rows =
-        fx::left_rows<3>(E, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic), __dmul_rn(fs.b1, fs.un),
-                         __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
+        fx::left_rows<3>(E, B0, B2, ea, eb, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic),
+                         __dmul_rn(fs.b1, fs.un), __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
     ok = ok && rows.emax < 2047;
     fx::i64 v[5];
+    const int as = sgn ? ea : 0, as1 = sgn ? eb : 0;
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
       const fx::u64 in[3] = {diff(sgn, 0, j), diff(sgn, 1, j), diff(sgn, 2, j)};
-      const fx::Proj p = fx::project<3>(rows, E, sgn ? ea : 0, in);
-      v[j] = q == 1 ? p.r - p.z : (q == 0 ? p.z + p.tc : p.z - p.tc);
+      const fx::Proj p = fx::project<3>(rows, E, as, as1, in);
+      v[j] = q == 1 ? fx::entropy<3>(rows, as, as1, p) : (q == 0 ? p.z + p.tc : p.z - p.tc);
     }
     bool wide;
     const ReconParams &rp = s_rp[q == 1 ? 0 : 1];
-    double h = field_lanes<AI>(v, s_sp.ka[0][q], rows.um + ea - 1592, ok, sgn, other, rp,
-                                         wide);
+    double h = field_lanes<AI>(v, s_sp.ka[0][q], (q == 1 ? rows.ue + eb : rows.um + ea) - 1592, ok,
+                               sgn, other, rp, wide);
     if (wide && act && sgn == 0)
       h = 6.0 * face_wide3<REG, AI>(
                                      pl, f, q, fs.un, fs.ic, fs.b1, fs.b2,
@@ -325,7 +326,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
         if constexpr (kPacked) {
           double hs[3];
           face_fields<3, AI>(
-              fs, s_sp.ka[0], s_sp.ea[0],
+              fs, s_sp.ka[0], s_sp.ea[0], s_sp.eb[0],
               [&](int s, int c, int j) {
                 return dp[(s ? (c == 0 ? 1 : 2 + c) : c) * ND + f + j];
               },
@@ -431,8 +432,11 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
   }
 }
 
+// Three blocks an SM for the Euler faces on the integer pipes: the compiler
+// would take 220 registers (two blocks; 64 x 1600 cells: 173 us a step, 151 with three).
 template <int NC, int AI, bool P1, int PREC, int R = 3>
-__global__ void __launch_bounds__(kThreads1D) k_line1d(const __grid_constant__ StageArgs a) {
+__global__ void __launch_bounds__(kThreads1D, (NC == 3 && R == 3 && P1 && PREC == 0) ? 3 : 0)
+    k_line1d(const __grid_constant__ StageArgs a) {
   extern __shared__ double sm[];
   pdl_start();
   line1d_tile<NC, AI, P1, PREC, kT1, R>(a, blockIdx.y, blockIdx.x,

@@ -273,7 +273,8 @@ struct ZA6Part {
   double num, den;  // f = v2 + num / (6 den)
 };
 
-template <int AI, bool P1>
+// EXACT: the deviation from the mean in FP64 (mu of eq. (22)) instead of FP32.
+template <int AI, bool P1, bool EXACT = false>
 __device__ __forceinline__ ZA6Part za6d(double d0, double d1, double d2, double d3, double d4,
                                         const ReconParams &P) {
   const double s0 = d1 - d0, s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3;
@@ -283,7 +284,15 @@ __device__ __forceinline__ ZA6Part za6d(double d0, double d1, double d2, double 
   const double t3 = fma(3.0, d4, -5.0 * d3);
   const double r5 = fma(3.0, s1 - s2, s3 - s0);
   double e;
-  if (AI) {
+  auto dev64 = [&]() {
+    const double a0 = -(d0 + d1), a1 = -d1, a3 = d2, a4 = d2 + d3, a5 = a4 + d4;
+    const double m = ((a0 + a1) + (a3 + a4) + a5) * (1.0 / 6.0);
+    return fabs(a0 - m) + fabs(a1 - m) + fabs(m) + fabs(a3 - m) + fabs(a4 - m) + fabs(a5 - m);
+  };
+  if (AI && EXACT) {
+    const double sm = fma(dev64(), P.me, P.mo);
+    e = sm * sm;
+  } else if (AI) {
     // deviations from v2, then from their mean, in FP32, on the differences
     // scaled by 2^(1019 - es) with es the largest of their exponents (so no
     // data range overflows FP32): dev = devf 2^(es - 1019)
@@ -296,11 +305,7 @@ __device__ __forceinline__ ZA6Part za6d(double d0, double d1, double d2, double 
     const float fm = ((fa0 + fa1) + (fa3 + fa4) + fa5) * (1.0f / 6.0f);
     const float devf = fabsf(fa0 - fm) + fabsf(fa1 - fm) + fabsf(fm) + fabsf(fa3 - fm) +
                        fabsf(fa4 - fm) + fabsf(fa5 - fm);
-    e = sens_term(devf, es, P, [&]() {
-      const double a0 = -(d0 + d1), a1 = -d1, a3 = d2, a4 = d2 + d3, a5 = a4 + d4;
-      const double m = ((a0 + a1) + (a3 + a4) + a5) * (1.0 / 6.0);
-      return fabs(a0 - m) + fabs(a1 - m) + fabs(m) + fabs(a3 - m) + fabs(a4 - m) + fabs(a5 - m);
-    });
+    e = sens_term(devf, es, P, dev64);
   } else {
     e = P.efix;
   }
@@ -394,19 +399,37 @@ __device__ __forceinline__ double pair_flux(double base, const ZA6Part &p, const
 }
 
 // The two reconstructions of one field in FP64 from its differences: the path
-// of p != 1, and of magnitudes the integer path leaves out (a field whose
-// largest difference is below 2^-959, below mu_0, or not finite).
+// of p != 1, and of what the integer path leaves out (magnitudes below 2^-959
+// or mu_0 or not finite, and differences too far apart: fx::uneven_fields).
+// za_wide: one of them, as a call (every lane layout makes the same one).  Where
+// the sensitivity term counts it has to be formed in FP64: beside a jump it is
+// what the weight of the candidates across the jump hangs on.
+template <int AI>
+__device__ __noinline__ ZA6Part za_wide(double d0, double d1, double d2, double d3, double d4,
+                                        const ReconParams &P) {
+  return za6d<(AI != kNoAi), true, (AI == kAi)>(d0, d1, d2, d3, d4, P);
+}
+// The differences of f^+ (sgn = 0) or of the mirrored f^- (1).
+__device__ __forceinline__ void split_differences(const double *dw, const double *dg, double A,
+                                                  int sgn, double (&d)[5]) {
+#pragma unroll
+  for (int j = 0; j < 5; ++j) d[j] = sgn ? fma(A, dw[4 - j], -dg[4 - j]) : fma(A, dw[j], dg[j]);
+}
+template <int AI, bool P1>
+__device__ __forceinline__ ZA6Part recon_wide(const double *dw, const double *dg, double A, int sgn,
+                                              const ReconParams &P) {
+  double d[5];
+  split_differences(dw, dg, A, sgn, d);
+  if constexpr (P1)
+    return za_wide<AI>(d[0], d[1], d[2], d[3], d[4], P);
+  else
+    return za6d<(AI != kNoAi), false>(d[0], d[1], d[2], d[3], d[4], P);
+}
 template <int AI, bool P1>
 __device__ __noinline__ double pair_wide(double base, const double *dw, const double *dg, double A,
                                          const ReconParams &P) {
-  double dp[5], dm[5];
-#pragma unroll
-  for (int j = 0; j < 5; ++j) {
-    dp[j] = fma(A, dw[j], dg[j]);
-    dm[4 - j] = fma(A, dw[j], -dg[j]);
-  }
-  return pair_flux(base, za6d<(AI != kNoAi), P1>(dp[0], dp[1], dp[2], dp[3], dp[4], P),
-                   za6d<(AI != kNoAi), P1>(dm[0], dm[1], dm[2], dm[3], dm[4], P));
+  const ZA6Part p = recon_wide<AI, P1>(dw, dg, A, 0, P), m = recon_wide<AI, P1>(dw, dg, A, 1, P);
+  return pair_flux(base, p, m);
 }
 
 // The sensitivity term of recon6 for one stencil (see there) in units of 2^k:
@@ -463,7 +486,7 @@ __device__ __forceinline__ double field_flux(const double (&dw)[5], const double
   const double base = __dsub_rn(centre, xw[2]);
   if constexpr (P1) {
     const int es = fx::top_exponent(xw, dg);
-    if (es >= P.es_lo && es <= P.es_hi) {
+    if (es >= P.es_lo && es <= P.es_hi && !fx::uneven(xw, dg, es, centre)) {
       fx::i64 x[5], g[5], c = 0;
 #pragma unroll
       for (int j = 0; j < 5; ++j) {
@@ -1158,28 +1181,62 @@ __device__ __forceinline__ double field_lanes(const fx::i64 (&v)[5], const fx::L
   return any == 0 ? 0.0 : fx::from_fixed(S, k);
 }
 
+// Left eigenvectors of a face for the integer path.
+template <int NC>
+__device__ __forceinline__ fx::LeftRows<NC> face_rows(const FaceState &fs, const int (&E)[NC],
+                                                      int B0, int B2, int a, int a1) {
+  return fx::left_rows<NC>(E, B0, B2, a, a1, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic),
+                           __dmul_rn(fs.b1, fs.un), __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
+}
+// Whether a face's differences are too far apart for the integer path; sl, sr:
+// sqrt(rho) of its two cells.  The second part is a call: few faces come to it.
+template <int NC>
+__device__ __forceinline__ unsigned strong_face(const FaceState &fs, const fx::LeftRows<NC> &rows,
+                                                int a, int a1, double sl, double sr) {
+  const int floor = fx::exponent(sl) + fx::exponent(sr) - fx::exponent(fs.ic) - 1023;
+  return fx::strong_fields<NC>(rows, a, a1, fs.ic, fs.ut, floor);
+}
+template <int NC, class Diff>
+__device__ __noinline__ bool uneven_call(Diff diff, unsigned strong, int a, int a1, int um, int ue,
+                                         int us, double b2, double b1, double un, double ut,
+                                         double ic) {
+  return (strong & fx::uneven_fields<NC>(diff, a, a1, um, ue, us, b2, b1, __dmul_rn(un, ic),
+                                         __dmul_rn(b1, un), __dmul_rn(b1, ut), ic, ut)) != 0;
+}
+template <int NC, class Diff>
+__device__ __forceinline__ bool uneven_face(const FaceState &fs, const fx::LeftRows<NC> &rows, int a,
+                                            int a1, double sl, double sr, Diff diff) {
+  const unsigned strong = strong_face<NC>(fs, rows, a, a1, sl, sr);
+  return strong != 0 && uneven_call<NC>(diff, strong, a, a1, rows.um, rows.ue, rows.us, fs.b2, fs.b1,
+                                        fs.un, fs.ut, fs.ic);
+}
+
 // 6 h of the fields of one face from its packed differences diff(s, q, j) of the
 // state (s = 0) and the physical flux (s = 1), component q, pair j; KA[m]: the fields' speeds
-// (fx::speed) with the exponents a (acoustic fields) and a1 (the others).
-template <int NC, int AI, class Diff, class Wide, class RP>
-__device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb *KA, int a, int a1,
-                                            Diff diff, RP rp, Wide wide, double (&h)[NC]) {
+// (fx::speed) with the exponents a (acoustic fields) and a1 (the others).  False: the face is
+// left to FP64 (differences not finite or too far apart, or a field out of range), which the
+// caller does in a call of its own when nothing else is live (here it cost 200 bytes of spills).
+template <int NC, int AI, class Diff, class RP>
+__device__ __forceinline__ bool face_fields(const FaceState &fs, double sl, double sr,
+                                           const fx::Limb *KA, int a, int a1, Diff diff, RP rp,
+                                           double (&h)[NC]) {
   int E[NC], B0, B2, top;
-  bool ok = face_exponents<NC>(a, a1, diff, E, B0, B2, top);
-  if (top == 0) {  // nothing varies over the stencil
+  const bool ok = face_exponents<NC>(a, a1, diff, E, B0, B2, top);
 #pragma unroll
-    for (int m = 0; m < NC; ++m) h[m] = 0.0;
-    return;
-  }
-  const fx::LeftRows<NC> rows =
-      fx::left_rows<NC>(E, B0, B2, a, a1, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic),
-                        __dmul_rn(fs.b1, fs.un), __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
-  ok = ok && rows.emax < 2047;
+  for (int m = 0; m < NC; ++m) h[m] = 0.0;
+  if (top == 0) return true;  // nothing varies over the stencil
+  const fx::LeftRows<NC> rows = face_rows<NC>(fs, E, B0, B2, a, a1);
+  if (!(ok && rows.emax < 2047) || uneven_face<NC>(fs, rows, a, a1, sl, sr, diff)) return false;
+  bool done = true;
   fx::i64 w[5], g[5];
   auto field = [&](int m, int k) {
     const FieldValue f = field_call<AI>(w[0], w[1], w[2], w[3], w[4], g[0], g[1], g[2], g[3], g[4],
                                         KA[m], k - 1592, rp(m));
-    h[m] = ok && !f.wide ? f.h6 : 6.0 * wide(m);
+    h[m] = f.h6;
+    if (f.wide) {  // (a branch that is kept holds the next field's sums behind this call: 255
+      done = false;  // registers without it, 196 with)
+      asm volatile("" ::: "memory");
+    }
   };
   if constexpr (NC == 4) {
 #pragma unroll
@@ -1217,6 +1274,7 @@ __device__ __forceinline__ void face_fields(const FaceState &fs, const fx::Limb 
   field(0, rows.um + a);
   part([](const fx::Proj &p) { return p.z - p.tc; });
   field(NC - 1, rows.um + a);
+  return done;
 }
 
 }  // namespace weno

@@ -10,7 +10,9 @@
 // rounding: it is homogeneous of degree one, its answer is an average of
 // candidates within the stencil's variation, and so an error of a few units
 // of 2^-57 of the largest difference, in every difference, is below the
-// rounding FP64 gives it (2^-53 per operation).
+// rounding FP64 gives it (2^-53 per operation) as long as the differences that
+// the weights choose are not far smaller than the largest.  Beside a strong
+// jump they can be; such faces are left to FP64 (uneven_fields).
 //
 // Measured at 2048^2, FP64, one step: 33.5 ms with the reconstruction and the
 // projections on the FP64 pipe, 16.0 ms with the reconstruction here, 9.16 ms
@@ -428,6 +430,81 @@ WENO_FX i64 project_shear(const LeftRows<4> &c, const int (&E)[4], int a, u64 rh
   return project_shear(c, E[0], a, rho, mt);
 }
 #endif
+
+// Where one unit a field is not enough.  The unit is 2^-57 of the stencil's
+// largest difference; the weights may choose a candidate whose differences are
+// far smaller, and FP64 holds those to 2^-53 of their own.  That shows only
+// where the unit is also above the rounding of the face's flux: h is off by a
+// few units in any case, and 2^-53 rho c of it by the rounding of the pressure.
+// So a field is left to FP64 where its scale is more than 2^kStrong rho c (the
+// shear field's, a momentum's: rho c times the larger of c and ut) and two adjacent
+// differences (three of the four candidates are made of two) are both more than
+// 2^kUneven below it, in the terms that they are sums of.  With 8 and 4 no
+// state tried (jumps of pressure and density up to 1e18, random cells up to
+// 1e12 apart) is further off than 2.4 times the FP64 formulas, as with 4 and 4;
+// of 3000 random pairs of states one in a hundred is off by 6 times (4: 2, 10:
+// 15).  Tubes and quadrants with pressures of 0.1 to 2 stay here (with 4 a few
+// faces did not, and as such a face takes its warp 20 us longer, a step of 64 x
+// 1600 cells took 210 us, 149 without them).
+constexpr int kStrong = 8, kUneven = 4;
+// Fields that may need FP64 as far as their scales tell, as a mask; floor: the
+// exponent of rho c, not biased.
+template <int NC>
+WENO_FX unsigned strong_fields(const LeftRows<NC> &c, int a, int a1, double ic, double ut, int floor) {
+  const int least = floor + kStrong + 1535;
+  unsigned m = c.um + a > least ? 1u | (1u << (NC - 1)) : 0u;
+  m |= c.ue + a1 > least ? 2u : 0u;
+  if (NC == 4) m |= c.us + a1 > least + imax(exponent(ut), 2046 - exponent(ic)) - 1023 ? 4u : 0u;
+  return m;
+}
+// Those of them with two adjacent small differences.
+template <int NC, class Diff>
+WENO_FX unsigned uneven_fields(Diff diff, int a, int a1, int um, int ue, int us, double b2,
+                               double b1, double t1, double t2, double t3, double ic, double ut) {
+  const int none = -65536, fu = exponent(ut);
+  const int c[4] = {imax(exponent(b2), exponent(t1)), imax(exponent(t2), exponent(ic)),
+                    NC == 4 ? exponent(t3) : exponent(b1), exponent(b1)};
+  int lz = none, le = none, ls = none;  // the pair before
+  unsigned m = 0;
+#pragma unroll 1
+  for (int j = 0; j < 5; ++j) {
+    int zu = none, zf = none, r0 = none, r2 = none;
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const int u = packed_exponent(diff(0, q, j)), f = packed_exponent(diff(1, q, j));
+      const int xu = u ? u : none, xf = f ? f : none;
+      zu = imax(zu, xu + c[q]);
+      zf = imax(zf, xf + c[q]);
+      if (q == 0) r0 = imax(xu, xf - a1);
+      if (NC == 4 && q == 2) r2 = imax(xu, xf - a1);
+    }
+    const int z = imax(zu, zf - a), e = imax(imax(zu, zf - a1), 1023 + r0), s = imax(fu + r0, 1023 + r2);
+    if (j > 0) {
+      if (imax(z, lz) < um - kUneven) m |= 1u | (1u << (NC - 1));
+      if (imax(e, le) < ue - kUneven) m |= 2u;
+      if (NC == 4 && imax(s, ls) < us - kUneven) m |= 4u;
+    }
+    lz = z;
+    le = e;
+    ls = s;
+  }
+  return m;
+}
+// The same for a scalar's ten differences with the largest exponent es, 2^kUneven
+// above the centre values (a scalar has no pressure whose rounding would cover
+// more).
+WENO_FX bool uneven(const double (&xw)[5], const double (&dg)[5], int es, double centre) {
+  if (es <= exponent(centre) + kUneven) return false;
+  bool m = false;
+  int last = 0;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const int e = imax(exponent(xw[j]), exponent(dg[j]));
+    m = m || (j > 0 && imax(e, last) < es - kUneven);
+    last = e;
+  }
+  return m;
+}
 
 // The stencil differences g + x of f^+ become those of the mirrored f^-:
 // x - g in reverse order.

@@ -429,12 +429,16 @@ __host__ __device__ constexpr size_t smem_euler2d_tma() {
 }
 
 // GLF speed of field m of nc (max|u| + c for every field in the single mode).
-__device__ __forceinline__ double field_speed(const StageArgs &a, const unsigned long long *al,
-                                              int m, int nc) {
+__device__ __forceinline__ double field_speed(int alpha_single, const unsigned long long *al, int m,
+                                              int nc) {
   unsigned long long v = al[m];
-  if (a.alpha_single)
+  if (alpha_single)
     for (int q = 0; q < nc; ++q) v = max(v, al[q]);
   return bits2d(v);
+}
+__device__ __forceinline__ double field_speed(const StageArgs &a, const unsigned long long *al,
+                                              int m, int nc) {
+  return field_speed(a.alpha_single, al, m, nc);
 }
 
 // One tile (tile index `tile` of problem b) of a 2D stage, run by one block.
@@ -631,40 +635,84 @@ __device__ __forceinline__ void make_speeds(const StageArgs &a, long long b, int
   }
 }
 
-// Field m of face (fr, fc) along DIR in FP64 from the staged cells (less its
-// centre values): what the integer path leaves out.
-template <int TX, int TY, int AI>
-__device__ __noinline__ double face_wide(const double *sm, int dir, int fr, int fc, int m, double un,
-                                         double ut, double ic, double b1, double b2, double A,
-                                         const ReconParams &rp) {
+// The offsets of face (fr, fc) along dir: its left cell in the box and the
+// planes, and the steps to the next cell.
+template <int TX, int TY>
+struct FaceAt {
+  using L = Tile6<TX, TY>;
+  int oL, kL, stB, stP;
+  __device__ __forceinline__ FaceAt(int dir, int fr, int fc) {
+    const int rL = fr + (dir ? L::R - 1 : L::R), cL = fc + (dir ? L::R : L::R - 1);
+    oL = rL * L::BW + cL + L::XO - L::R;
+    kL = rL * L::W + cL;
+    stB = dir ? L::BW : 1;
+    stP = dir ? L::W : 1;
+  }
+};
+// The packed differences of a face for the integer path.
+template <int ND>
+struct PackedFace {
+  const fx::u64 *pf;
+  int ps;
+  __device__ __forceinline__ fx::u64 operator()(int s, int q, int j) const {
+    return pf[(s ? (q == 0 ? 1 : 3 + q) : q) * ND + j * ps];
+  }
+};
+// 2 F_hat of a face from its fields' 6 h: F_L + F_R and a twelfth of what
+// backproject4 gives.
+template <int TX, int TY>
+__device__ __forceinline__ void face_flux6(const double *sm, int dir, const FaceAt<TX, TY> &at,
+                                           const FaceState &fs, const double (&h)[4], double *out) {
   using L = Tile6<TX, TY>;
   const double *const box = sm + L::kBox, *const pl = sm + L::kPl;
-  FaceState fs = {};
-  fs.un = un;
-  fs.ut = ut;
-  fs.ic = ic;
-  fs.b1 = b1;
-  fs.b2 = b2;
-  double U[2][4], F[2][4], dw[5], dg[5];
+  const double *const bn = box + (1 + dir) * L::PB, *const bt = box + (2 - dir) * L::PB;
+  const double *const un = pl + (1 + dir) * L::REG, *const H = pl + 3 * L::REG;
+  const int oL = at.oL, oR = oL + at.stB, kL = at.kL, kR = kL + at.stP;
+  double F0, F1, F2, F3, FL1, FL2, FL3, FR1, FR2, FR3;
+  backproject4(fs, h[0], h[1], h[2], h[3], F0, F1, F2, F3);
+  const double mnL = bn[oL], mnR = bn[oR];
+  normal_flux(box[oL], mnL, bt[oL], box[3 * L::PB + oL], un[kL], H[kL], FL1, FL2, FL3);
+  normal_flux(box[oR], mnR, bt[oR], box[3 * L::PB + oR], un[kR], H[kR], FR1, FR2, FR3);
+  out[0] = fma(1.0 / 12.0, F0, mnL + mnR);
+  out[1 + dir] = fma(1.0 / 12.0, F1, FL1 + FR1);
+  out[2 - dir] = fma(1.0 / 12.0, F2, FL2 + FR2);
+  out[3] = fma(1.0 / 12.0, F3, FL3 + FR3);
+}
+// Face (fr, fc) along dir with all its fields in FP64 from the staged cells: what
+// the integer path leaves out.  al: its speed maxima.
+template <int TX, int TY, int AI>
+__device__ __noinline__ void face_wide(double *sm, int dir, int fr, int fc, FaceState fs,
+                                       const unsigned long long *al, int alpha_single,
+                                       const SchemeParams &scheme) {
+  using L = Tile6<TX, TY>;
+  const double *const box = sm + L::kBox, *const pl = sm + L::kPl;
+  const double *const un = pl + (1 + dir) * L::REG, *const H = pl + 3 * L::REG;
+  const FaceAt<TX, TY> at(dir, fr, fc);
+  double U[2][4], F[2][4], dw[4][5], dg[4][5], h[4];
+#pragma unroll
   for (int j = 0; j < 6; ++j) {
-    const int r = dir ? fr + j : 3 + fr, c = dir ? 3 + fc : fc + j;
-    const int o = r * L::BW + c + L::XO - 3, k = r * L::W + c;
+    const int o = at.oL + (j - 2) * at.stB, k = at.kL + (j - 2) * at.stP;
     double *const u = U[j & 1], *const f = F[j & 1];
     u[0] = box[o];
     u[1] = f[0] = box[(1 + dir) * L::PB + o];
     u[2] = box[(2 - dir) * L::PB + o];
     u[3] = box[3 * L::PB + o];
-    normal_flux(u[0], u[1], u[2], u[3], pl[(1 + dir) * L::REG + k], pl[3 * L::REG + k], f[1], f[2],
-                f[3]);
+    normal_flux(u[0], u[1], u[2], u[3], un[k], H[k], f[1], f[2], f[3]);
     if (j == 0) continue;
     const double *const u0 = U[(j - 1) & 1], *const f0 = F[(j - 1) & 1];
-    double w[4], g[4];
-    project4(fs, u[0] - u0[0], u[1] - u0[1], u[2] - u0[2], u[3] - u0[3], w[0], w[1], w[2], w[3]);
-    project4(fs, f[0] - f0[0], f[1] - f0[1], f[2] - f0[2], f[3] - f0[3], g[0], g[1], g[2], g[3]);
-    dw[j - 1] = w[m];
-    dg[j - 1] = g[m];
+    project4(fs, u[0] - u0[0], u[1] - u0[1], u[2] - u0[2], u[3] - u0[3], dw[0][j - 1], dw[1][j - 1],
+             dw[2][j - 1], dw[3][j - 1]);
+    project4(fs, f[0] - f0[0], f[1] - f0[1], f[2] - f0[2], f[3] - f0[3], dg[0][j - 1], dg[1][j - 1],
+             dg[2][j - 1], dg[3][j - 1]);
   }
-  return pair_wide<AI, true>(-A * dw[2], dw, dg, A, rp);
+#pragma unroll 1
+  for (int m = 0; m < 4; ++m) {
+    const double A = field_speed(alpha_single, al, m, 4);
+    h[m] = 6.0 * pair_wide<AI, true>(-A * dw[m][2], dw[m], dg[m], A,
+                                     scheme.rp[m == 0 || m == 3 ? 1 : 0]);
+  }
+  double *const out = sm + (dir ? L::kFy + (fr * TX + fc) * 4 : L::kFx + (fr * (TX + 1) + fc) * 4);
+  face_flux6<TX, TY>(sm, dir, at, fs, h, out);
 }
 
 // One direction (0: x, 1: y) of a tile.  The direction is a run-time value: the
@@ -736,23 +784,22 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long lo
     const int p0 = fr * lp + fc;
     const int rL = fr + (dir ? R - 1 : R), cL = fc + (dir ? R : R - 1);
     const int kL = rL * W + cL, kR = kL + stP;
-    const int oL = bo(rL, cL), oR = oL + stB;
+    const int oL = bo(rL, cL);
     FaceState fs;
     if (!roe_face(pl[kL], un[kL], ut[kL], pl[3 * REG + kL], pl[kR], un[kR], ut[kR],
                   pl[3 * REG + kR], gm1, fs))
       record_status(a.status, 3, a.stage, b, j0 + fr, i0 + fc);
     double h[4];
+    double *const out = fo + (fr * lf + fc) * 4;
     if constexpr (kPacked) {
-      const fx::u64 *const pf = dp + p0;
-      face_fields<4, AI>(
-          fs, sp.ka[dir], sp.ea[dir], sp.eb[dir],
-          [&](int s, int q, int j) { return pf[(s ? (q == 0 ? 1 : 3 + q) : q) * ND + j * ps]; },
-          [&](int m) -> const ReconParams & { return (m == 0 || m == 3) ? rp4 : rp2; },
-          [&](int m) {
-            return face_wide<TX, TY, AI>(sm, dir, fr, fc, m, fs.un, fs.ut, fs.ic, fs.b1, fs.b2,
-                                         field_speed(a, al, m, 4), (m == 0 || m == 3) ? rp4 : rp2);
-          },
-          h);
+      const PackedFace<ND> diff = {dp + p0, ps};
+      const bool done = face_fields<4, AI>(
+          fs, pl[kL], pl[kR], sp.ka[dir], sp.ea[dir], sp.eb[dir], diff,
+          [&](int m) -> const ReconParams & { return (m == 0 || m == 3) ? rp4 : rp2; }, h);
+      if (done)
+        face_flux6<TX, TY>(sm, dir, FaceAt<TX, TY>(dir, fr, fc), fs, h, out);
+      else
+        face_wide<TX, TY, AI>(sm, dir, fr, fc, fs, al, a.alpha_single, scheme);
     } else {
       double dw[4][5], dg[4][5];
 #pragma unroll
@@ -772,38 +819,17 @@ __device__ __forceinline__ void tile6_sweep(const StageArgs &a, int dir, long lo
         else
           h[m] = field_flux<AI, P1>(dw[m], dg[m], A, (m == 0 || m == 3) ? rp4 : rp2, 0.0);
       }
-    }
-    double F0, F1, F2, F3;
-    backproject4(fs, h[0], h[1], h[2], h[3], F0, F1, F2, F3);
-    // the centre values.  Packed: the faces hold 2 F_hat, F_L + F_R and a twelfth
-    // of what backproject4 gives from the fields' 6 h; else 4 F_hat, with
-    // 2 (F_L + F_R) = 4 F_L + 2 dF of the centre pair.
-    {
+      // the centre values: 4 F_hat += 2 (F_L + F_R) = 4 F_L + 2 dF of the centre pair
+      double F0, F1, F2, F3, FL1, FL2, FL3;
+      backproject4(fs, h[0], h[1], h[2], h[3], F0, F1, F2, F3);
+      const int pc = p0 + 2 * ps;
       const double mnL = bn[oL];
-      double FL1, FL2, FL3;
       normal_flux(box[oL], mnL, bt[oL], box[3 * PB + oL], un[kL], pl[3 * REG + kL], FL1, FL2, FL3);
-      if constexpr (kPacked) {
-        const double mnR = bn[oR];
-        double FR1, FR2, FR3;
-        normal_flux(box[oR], mnR, bt[oR], box[3 * PB + oR], un[kR], pl[3 * REG + kR], FR1, FR2,
-                    FR3);
-        F0 = fma(1.0 / 12.0, F0, mnL + mnR);
-        F1 = fma(1.0 / 12.0, F1, FL1 + FR1);
-        F2 = fma(1.0 / 12.0, F2, FL2 + FR2);
-        F3 = fma(1.0 / 12.0, F3, FL3 + FR3);
-      } else {
-        const int pc = p0 + 2 * ps;
-        F0 = fma(4.0, mnL, fma(2.0, dd[ND + pc], F0));
-        F1 = fma(4.0, FL1, fma(2.0, dd[4 * ND + pc], F1));
-        F2 = fma(4.0, FL2, fma(2.0, dd[5 * ND + pc], F2));
-        F3 = fma(4.0, FL3, fma(2.0, dd[6 * ND + pc], F3));
-      }
+      out[0] = fma(4.0, mnL, fma(2.0, dd[ND + pc], F0));
+      out[1 + dir] = fma(4.0, FL1, fma(2.0, dd[4 * ND + pc], F1));
+      out[2 - dir] = fma(4.0, FL2, fma(2.0, dd[5 * ND + pc], F2));
+      out[3] = fma(4.0, FL3, fma(2.0, dd[6 * ND + pc], F3));
     }
-    double *out = fo + (fr * lf + fc) * 4;
-    out[0] = F0;
-    out[1 + dir] = F1;
-    out[2 - dir] = F2;
-    out[3] = F3;
   }
   __syncthreads();
 }

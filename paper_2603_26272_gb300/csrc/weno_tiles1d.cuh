@@ -31,18 +31,12 @@ __device__ __forceinline__ void add_centre3(const double (*pl)[REG], const doubl
   }
 }
 
-// Field m of face f in FP64 from the staged cells (less its centre values):
-// what the integer path leaves out.
-template <int REG, int AI>
-__device__ __noinline__ double face_wide3(const double (*pl)[REG], int f, int m, double un,
-                                          double ic, double b1, double b2, double A,
-                                          const ReconParams &rp) {
-  FaceState fs = {};
-  fs.un = un;
-  fs.ic = ic;
-  fs.b1 = b1;
-  fs.b2 = b2;
-  double dw[5], dg[5];
+// The projected differences of field m of face f in FP64 from the staged cells.
+template <int REG>
+__device__ __forceinline__ void wide_differences3(const double (*pl)[REG], int f, int m,
+                                                  const FaceState &fs, double (&dw)[5],
+                                                  double (&dg)[5]) {
+#pragma unroll
   for (int j = 0; j < 5; ++j) {
     const int k = f + j;
     dw[j] = project3_field(fs, m, pl[0][k + 1] - pl[0][k], pl[1][k + 1] - pl[1][k],
@@ -50,7 +44,38 @@ __device__ __noinline__ double face_wide3(const double (*pl)[REG], int f, int m,
     dg[j] = project3_field(fs, m, pl[6][k + 1] - pl[6][k], pl[7][k + 1] - pl[7][k],
                            pl[8][k + 1] - pl[8][k]);
   }
-  return pair_wide<AI, true>(-A * dw[2], dw, dg, A, rp);
+}
+// The packed differences of a face for the integer path.
+template <int ND>
+struct PackedFace3 {
+  const fx::u64 *pf;
+  __device__ __forceinline__ fx::u64 operator()(int s, int q, int j) const {
+    return pf[(s ? (q == 0 ? 1 : 2 + q) : q) * ND + j];
+  }
+};
+// Face f with all its fields in FP64 from the staged cells: what the integer
+// path leaves out.  al: the speed maxima; out: the face.
+template <int REG, int AI>
+__device__ __noinline__ void face_wide3(const double (*pl)[REG], int f, double gm1,
+                                        const unsigned long long *al, int alpha_single,
+                                        const SchemeParams &scheme, double *out) {
+  FaceState fs = {};
+  const int kL = f + 2, kR = f + 3;
+  roe_face(pl[5][kL], pl[3][kL], 0.0, pl[4][kL], pl[5][kR], pl[3][kR], 0.0, pl[4][kR], gm1, fs);
+  double h[3];
+#pragma unroll 1
+  for (int m = 0; m < 3; ++m) {
+    double dw[5], dg[5];
+    const double A = field_speed(alpha_single, al, m, 3);
+    wide_differences3<REG>(pl, f, m, fs, dw, dg);
+    h[m] = 6.0 * pair_wide<AI, true>(-A * dw[2], dw, dg, A, scheme.rp[m == 1 ? 0 : 1]);
+  }
+  double F0, F1, F2;
+  backproject3(fs, h[0], h[1], h[2], F0, F1, F2);
+  add_centre3<REG>(pl, nullptr, 0, kL, F0, F1, F2);
+  out[0] = F0;
+  out[1] = F1;
+  out[2] = F2;
 }
 
 // Lanes per face of the latency layout and its cells per 128-thread tile: a
@@ -201,32 +226,46 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     if (!roe_face(pl[5][kL], pl[3][kL], 0.0, pl[4][kL], pl[5][kR], pl[3][kR], 0.0, pl[4][kR], gm1,
                   fs) && act && r == 0)
       record_status(a.status, 3, a.stage, b, 0, i0 + f);
-    auto diff = [&](int s, int c, int j) {
-      return dp[(s ? (c == 0 ? 1 : 2 + c) : c) * ND + f + j];
-    };
+    const PackedFace3<ND> diff = {dp + f};
     int E[3], B0, B2, top;
     const int ea = s_sp.ea[0], eb = s_sp.eb[0];
-    bool ok = face_exponents<3>(ea, eb, diff, E, B0, B2, top);
-    const fx::LeftRows<3> rows =
-        fx::left_rows<3>(E, B0, B2, ea, eb, fs.b2, fs.b1, __dmul_rn(fs.un, fs.ic),
-                         __dmul_rn(fs.b1, fs.un), __dmul_rn(fs.b1, fs.ut), fs.ic, fs.ut);
-    ok = ok && rows.emax < 2047;
-    fx::i64 v[5];
-    const int as = sgn ? ea : 0, as1 = sgn ? eb : 0;
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-      const fx::u64 in[3] = {diff(sgn, 0, j), diff(sgn, 1, j), diff(sgn, 2, j)};
-      const fx::Proj p = fx::project<3>(rows, E, as, as1, in);
-      v[j] = q == 1 ? fx::entropy<3>(rows, as, as1, p) : (q == 0 ? p.z + p.tc : p.z - p.tc);
-    }
-    bool wide;
+    const bool in = face_exponents<3>(ea, eb, diff, E, B0, B2, top);
+    const fx::LeftRows<3> rows = face_rows<3>(fs, E, B0, B2, ea, eb);
+    // all fields of a face that has one left to FP64 go there (face_wide3); a
+    // warp of such faces skips the integer path
+    const bool ok = in && rows.emax < 2047 &&
+                    (top == 0 || !uneven_face<3>(fs, rows, ea, eb, pl[5][kL], pl[5][kR], diff));
     const ReconParams &rp = s_rp[q == 1 ? 0 : 1];
-    double h = field_lanes<AI>(v, s_sp.ka[0][q], (q == 1 ? rows.ue + eb : rows.um + ea) - 1592, ok,
-                               sgn, other, rp, wide);
-    if (wide && act && sgn == 0)
-      h = 6.0 * face_wide3<REG, AI>(
-                                     pl, f, q, fs.un, fs.ic, fs.b1, fs.b2,
-                                     field_speed(a, a.alpha_in + b * 8, q, 3), rp);
+    bool wide = !ok;
+    double h = 0.0;
+    if (__any_sync(0xffffffffu, ok)) {
+      fx::i64 v[5];
+      const int as = sgn ? ea : 0, as1 = sgn ? eb : 0;
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const fx::u64 d[3] = {diff(sgn, 0, j), diff(sgn, 1, j), diff(sgn, 2, j)};
+        const fx::Proj p = fx::project<3>(rows, E, as, as1, d);
+        v[j] = q == 1 ? fx::entropy<3>(rows, as, as1, p) : (q == 0 ? p.z + p.tc : p.z - p.tc);
+      }
+      const int k0 = (q == 1 ? rows.ue + eb : rows.um + ea) - 1592;
+      h = field_lanes<AI>(v, s_sp.ka[0][q], k0, ok, sgn, other, rp, wide);
+    }
+    const unsigned todo = __ballot_sync(0xffffffffu, wide);
+    if (todo != 0) {
+      const bool mine = (todo >> (l - r) & 63u) != 0;
+      ZA6Part part = {0.0, 1.0};
+      double base = 0.0;
+      if (mine) {
+        double dw[5], dg[5];
+        const double A = field_speed(a, a.alpha_in + b * 8, q, 3);
+        wide_differences3<REG>(pl, f, q, fs, dw, dg);
+        base = -A * dw[2];
+        part = recon_wide<AI, true>(dw, dg, A, sgn, rp);
+      }
+      const ZA6Part mate = {__shfl_sync(0xffffffffu, part.num, other),
+                            __shfl_sync(0xffffffffu, part.den, other)};
+      if (mine && sgn == 0) h = 6.0 * pair_flux(base, part, mate);
+    }
     const double h1 = __shfl_sync(0xffffffffu, h, min(lane + 1, 31)),
                  h2 = __shfl_sync(0xffffffffu, h, min(lane + 2, 31));
     if (act && r == 0) {
@@ -240,14 +279,15 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
   } else if constexpr (LANES == 2) {
     // the positive (even lane) and the mirrored negative flux (odd lane) of a
     // scalar face, the operations of field_flux: the corrections meet by a lane
-    // shuffle; a face off the integer path is left to the even lane alone
+    // shuffle, and so do the FP64 parts where a face of the warp needs those
     const int f = tid >> 1, sgn = tid & 1;
     const bool act = (f <= T) && (i0 + f - 1 < nx);
     double dw[5] = {}, dg[5] = {}, xw[5] = {};
-    double A = 0.0, centre = 0.0;
-    int es = 0;
+    double A = 0.0, base = 0.0;
+    bool fixed = false, flat = false;
     fx::i64 c = 0;
     const ReconParams &rp = s_rp[0];
+    double scale = 0.0;
     if (act) {
       A = scalar_alpha_of(a.system, a.adv_speed, a.ustar, a.alpha_in + b * 8);
 #pragma unroll
@@ -256,29 +296,43 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
         dg[j] = pl[1][f + j + 1] - pl[1][f + j];
         xw[j] = __dmul_rn(A, dw[j]);
       }
-      centre = pl[1][f + 2] + pl[1][f + 3];
-      es = fx::top_exponent(xw, dg);
-    }
-    const bool fixed = P1 && act && es >= rp.es_lo && es <= rp.es_hi;
-    if (fixed) {
-      fx::i64 d[5];
+      const double centre = pl[1][f + 2] + pl[1][f + 3];
+      base = __dsub_rn(centre, xw[2]);
+      if constexpr (P1) {
+        const int es = fx::top_exponent(xw, dg);
+        fixed = es >= rp.es_lo && es <= rp.es_hi && !fx::uneven(xw, dg, es, centre);
+        if (fixed) {
+          fx::i64 d[5];
 #pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        const fx::i64 x = fx::to_fixed(xw[j], es), g = fx::to_fixed(dg[j], es);
-        if (sgn)
-          d[4 - j] = x - g;
-        else
-          d[j] = x + g;
+          for (int j = 0; j < 5; ++j) {
+            const fx::i64 x = fx::to_fixed(xw[j], es), g = fx::to_fixed(dg[j], es);
+            if (sgn)
+              d[4 - j] = x - g;
+            else
+              d[j] = x + g;
+          }
+          c = recon_fixed<AI>(d, es - 1079, rp);
+          scale = fx::scale_back(es);
+        } else {
+          unsigned long long any = 0;
+#pragma unroll
+          for (int j = 0; j < 5; ++j)
+            any |= (unsigned long long)(__double_as_longlong(xw[j]) | __double_as_longlong(dg[j])) << 1;
+          flat = any == 0;
+        }
       }
-      c = recon_fixed<AI>(d, es - 1079, rp);
     }
     c += __shfl_xor_sync(0xffffffffu, c, 1);
-    if (act && sgn == 0) {
-      if (fixed)
-        fl[f][0] = __fma_rn((double)c, fx::scale_back(es), __dsub_rn(centre, xw[2]));
-      else
-        fl[f][0] = field_flux<AI, P1>(dw, dg, A, rp, centre);
+    double h = flat ? base : __fma_rn((double)c, scale, base);
+    const bool wide = act && !fixed && !flat;
+    if (__any_sync(0xffffffffu, wide)) {
+      ZA6Part part = {0.0, 1.0};
+      if (wide) part = recon_wide<AI, P1>(dw, dg, A, sgn, rp);
+      const ZA6Part mate = {__shfl_xor_sync(0xffffffffu, part.num, 1),
+                            __shfl_xor_sync(0xffffffffu, part.den, 1)};
+      if (wide) h = pair_flux(base, part, mate);
     }
+    if (act && sgn == 0) fl[f][0] = h;
   } else {
     const int f = tid;  // face between cells i0+f-1 and i0+f; stencil f..f+2R-1
     if (f <= T && i0 + f - 1 < nx) {
@@ -323,20 +377,12 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
         const double A1 = field_speed(a, al, 0, 3), A2 = field_speed(a, al, 1, 3),
                      A3 = field_speed(a, al, 2, 3);
         double h1, h2, h3;
+        bool done = true;
         if constexpr (kPacked) {
           double hs[3];
-          face_fields<3, AI>(
-              fs, s_sp.ka[0], s_sp.ea[0], s_sp.eb[0],
-              [&](int s, int c, int j) {
-                return dp[(s ? (c == 0 ? 1 : 2 + c) : c) * ND + f + j];
-              },
-              [&](int m) -> const ReconParams & { return s_rp[m == 1 ? 0 : 1]; },
-              [&](int m) {
-                return face_wide3<REG, AI>(pl, f, m, fs.un, fs.ic, fs.b1, fs.b2,
-                                                     field_speed(a, al, m, 3),
-                                                     s_rp[m == 1 ? 0 : 1]);
-              },
-              hs);
+          done = face_fields<3, AI>(
+              fs, pl[5][kL], pl[5][kR], s_sp.ka[0], s_sp.ea[0], s_sp.eb[0], PackedFace3<ND>{dp + f},
+              [&](int m) -> const ReconParams & { return s_rp[m == 1 ? 0 : 1]; }, hs);
           h1 = hs[0];
           h2 = hs[1];
           h3 = hs[2];
@@ -385,6 +431,8 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
         fl[f][0] = F0;
         fl[f][1] = F1;
         fl[f][2] = F2;
+        if constexpr (kPacked)
+          if (!done) face_wide3<REG, AI>(pl, f, gm1, al, a.alpha_single, s_scheme, &fl[f][0]);
       }
     }
   }

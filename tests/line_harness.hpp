@@ -173,6 +173,14 @@ void fields_fixed(const Line<NC> &s, const Cell<double> *x, const Face<double> &
   if (top == 0) return;
   const LeftRows<NC> rows =
       left_rows<NC>(E, B0, B2, a, a1, f.b2, f.b1, f.un * f.ic, f.b1 * f.un, f.b1 * f.ut, f.ic, f.ut);
+  // fields left to FP64
+  const int floor = exponent(std::sqrt(x[2].rho)) + exponent(std::sqrt(x[3].rho)) - exponent(f.ic) - 1023;
+  unsigned left = strong_fields<NC>(rows, a, a1, f.ic, f.ut, floor);
+  if (left)
+    left &= uneven_fields<NC>([&](int k, int q, int j) { return P[k][q][j]; }, a, a1, rows.um, rows.ue,
+                              rows.us, f.b2, f.b1, f.un * f.ic, f.b1 * f.un, f.b1 * f.ut, f.ic, f.ut);
+  double wide[NC];
+  if (left) fields<double, NC>(s, x, f, A, i0, wide);
   i64 d[2][NC][5];
   for (int k = 0; k < 2; ++k)
     for (int j = 0; j < 5; ++j) {
@@ -188,6 +196,10 @@ void fields_fixed(const Line<NC> &s, const Cell<double> *x, const Face<double> &
   for (int m = 0; m < NC; ++m) {
     const bool slow = m > 0 && m < NC - 1;
     const int k0 = (!slow ? rows.um + a : m == 1 ? rows.ue + a1 : rows.us + a1) - 1592;
+    if (left >> m & 1) {
+      h[m] = wide[m];
+      continue;
+    }
     i64 *w = d[0][m], *g = d[1][m], X[5], G[5], p[5], n[5];
     for (int j = 0; j < 5; ++j) {
       X[j] = times_speed(speed(A[m], slow ? a1 : a), w[j]);

@@ -113,10 +113,12 @@ weno_status weno_wavespeeds(const weno_desc *d, const double *U, double *alpha, 
  * result; weights other than the default ones -- ai = 0, a larger epsilon or
  * mu0, p != 1 -- have three of them, for which the other numbers stand).  The
  * first such call on a new problem shape (nx, ny, nbatch,
- * precision, ai, p == 1) in a process times them on the caller's data: two
+ * precision, ai, p == 1, and in FP64 with ai = 1 and p = 1 whether eps <= 2^-126
+ * and mu0 <= 2^-100) in a process times them on the caller's data: two
  * launches of each shape on `stream`, writing only the workspace, with CUDA
  * events, and it synchronises the stream before it returns.  Later calls on
- * that shape are asynchronous as stated.  The environment variable
+ * that shape are asynchronous as stated; inside a stream capture a choice made
+ * for the other eps and mu0 serves too.  The environment variable
  * WENO_TILE2D = 0..10 forces one shape and skips the timing (use it when the
  * first call must not synchronise, e.g. inside a stream capture). */
 

@@ -314,11 +314,27 @@ weno_status choose_tile(const Ctx &c, const double *U, const unsigned long long 
     *out = forced;
     return WENO_OK;
   }
-  const auto key = std::make_tuple((long long)d->nx, (long long)d->ny, (long long)d->nbatch,
-                                   (int)d->precision, (int)d->ai, (int)(d->p == 1.0));
+  // One entry per kernel: the default weights (FP64, p = 1) have one of their own.
+  const int weights = weno::weight_mode(d->ai != 0, d->eps, d->mu0);
+  const int mode = weights == weno::kAiTiny && (d->precision == WENO_PREC_FP32_RECON || d->p != 1.0)
+                       ? (int)weno::kAi : weights;
+  const auto key_of = [&](int m) {
+    return std::make_tuple((long long)d->nx, (long long)d->ny, (long long)d->nbatch,
+                           (int)d->precision, m, (int)(d->p == 1.0));
+  };
+  const auto key = key_of(mode);
+  // Nothing can be timed inside a stream capture: there the choice made for the
+  // other weights with Ai on this grid stands in.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune.find(key);
+    if (it == g_tune.end() && mode != weno::kNoAi) {
+      if (cudaStreamIsCapturing(c.s, &capture) != cudaSuccess)
+        cudaGetLastError();  // (the legacy stream beside another's capture: reported by the launches)
+      else if (capture == cudaStreamCaptureStatusActive)
+        it = g_tune.find(key_of(mode == weno::kAi ? weno::kAiTiny : weno::kAi));
+    }
     if (it != g_tune.end()) {
       *out = it->second;
       return WENO_OK;
@@ -339,8 +355,7 @@ weno_status choose_tile(const Ctx &c, const double *U, const unsigned long long 
   int best = 0;
   float best_ms = 0.0f;
   weno_status st = WENO_OK;
-  const bool all = weno::all_tile_shapes(weno::weight_mode(d->ai != 0, d->eps, d->mu0), d->p == 1.0,
-                                         d->precision);
+  const bool all = weno::all_tile_shapes(weights, d->p == 1.0, d->precision);
   for (int v = 0; v < weno::kTileVariants && st == WENO_OK; ++v) {
     if (weno::tile_shape_built(all, v) != v) continue;  // runs as another shape
     a.tile_variant = v;

@@ -457,11 +457,12 @@ __device__ __forceinline__ fx::Flt sens_fixed(const fx::i64 (&d)[5], int k,
 }
 
 template <int AI>
-__device__ __forceinline__ fx::i64 recon_fixed(const fx::i64 (&d)[5], int k, const ReconParams &P) {
+__device__ __forceinline__ fx::i64 recon_fixed(const fx::i64 (&d)[5], int k, const ReconParams &P,
+                                               bool *lost = nullptr) {
   if constexpr (AI == kAiTiny)
-    return fx::recon6<false>(d[0], d[1], d[2], d[3], d[4], P.e3);
+    return fx::recon6<false>(d[0], d[1], d[2], d[3], d[4], P.e3, lost);
   else
-    return fx::recon6<true>(d[0], d[1], d[2], d[3], d[4], sens_fixed<AI>(d, k, P));
+    return fx::recon6<true>(d[0], d[1], d[2], d[3], d[4], sens_fixed<AI>(d, k, P), lost);
 }
 
 // One field of one face (FP64) from the differences dw[j] = w_{j+1} - w_j,
@@ -493,6 +494,7 @@ __device__ __forceinline__ double field_flux(const double (&dw)[5], const double
         x[j] = fx::to_fixed(xw[j], es);
         g[j] = fx::to_fixed(dg[j], es);
       }
+      if (fx::lost_pair(x, g)) return pair_wide<AI, P1>(base, dw, dg, A, P);
 #pragma unroll 1
       for (int s = 0; s < 2; ++s) {
         fx::i64 d[5];
@@ -1081,8 +1083,10 @@ __device__ __noinline__ FieldSum rough_call(fx::i64 x0, fx::i64 x1, fx::i64 x2, 
   if (!in_range(k + 57, P)) return FieldSum{0, INT_MIN};
   fx::shift_field(x, n);
   fx::shift_field(g, n);
-  return FieldSum{fx::rough_sum(x, g, [&](const fx::i64(&d)[5]) { return recon_fixed<AI>(d, k, P); }),
-                  k};
+  bool lost = false;
+  const fx::i64 S =
+      fx::rough_sum(x, g, [&](const fx::i64(&d)[5]) { return recon_fixed<AI>(d, k, P, &lost); });
+  return FieldSum{S, lost ? INT_MIN : k};
 }
 // 6 h of one field less its centre values; wide: the field is left to FP64.
 struct FieldValue {
@@ -1173,7 +1177,7 @@ __device__ __forceinline__ double field_lanes(const fx::i64 (&v)[5], const fx::L
       if (sgn) fx::mirror(y, f);
 #pragma unroll
       for (int j = 0; j < 5; ++j) d[j] = y[j] + f[j];
-      r = recon_fixed<AI>(d, k, P) - 3 * d[2];
+      r = recon_fixed<AI>(d, k, P, &wide) - 3 * d[2];
     }
   }
   r += shfl64(r, other);

@@ -100,6 +100,7 @@ WENO_FX double bitsd(u64 b) {
 
 WENO_FX uint32_t lo32(u64 x) { return (uint32_t)x; }
 WENO_FX uint32_t hi32(u64 x) { return (uint32_t)(x >> 32); }
+WENO_FX int imax(int a, int b) { return a > b ? a : b; }
 WENO_FX u64 abs64(i64 x) { return x < 0 ? 0 - (u64)x : (u64)x; }
 
 // a b / 2^64, low by at most 2 (the product of the low words and the carries
@@ -191,8 +192,13 @@ WENO_FX Flt normal_plus(u64 raw, int e, const Flt &s) {
 // wherever mu_0 is below the largest difference, and it could only decide
 // between candidates that agree to a few units; it is then left out, and an
 // indicator that is 0 in these units counts as 2^-4.
+// Where one is 0 (three equal cells: d0 = d1 = 0, d1 = d2 = 0 or d2 = d3 = 0) the
+// others' weights are 2^-4 / T of its own at most, below a unit of the candidates
+// from |r5| = 2^29 on.  Below (cubic data to its rounding) the weights hang on
+// the sensitivity term and on what the units leave of r5: *lost, for FP64 to take
+// over, whose differences of equal cells are 0 and the others' exact.
 template <bool SENS>
-WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e) {
+WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e, bool *lost = nullptr) {
   const i64 s0 = d1 - d0, s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3;
   const Ind i0 = indicator(s0, 2 * d1 + s0);           // t_0 = 3 d1 - d0
   const Ind i1 = indicator(s1, d1 + d2);               // t_1
@@ -220,6 +226,7 @@ WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e) {
   // T = 12 r5^2
   const u64 ra = abs64(r5);
   const int nt = clz64(ra) - 1;
+  if (lost && nt > 33 && nm < 62 && imax(imax(i0.n, i1.n), i2.n) == 62) *lost = true;
   const u64 sq = sqrhi(shl(ra, nt));
   const Flt T = normal(3ull * sq, ra ? 66 - 2 * nt : -16384);  // 0: far below every b_k
   // y_k = D_k z_k with the largest of D_k / b_k and 8 / T in [2^60, 2^61)
@@ -240,6 +247,25 @@ WENO_FX i64 recon6(i64 d0, i64 d1, i64 d2, i64 d3, i64 d4, const Flt &e) {
   const i64 Ns = (i64)(N - ((y0 + y2 + y3) >> 1));
   const u64 c = mulhi64(abs64(Ns), rcp64(shl(den, nd)));
   return (d1 + 2 * d2) + (Ns < 0 ? -(i64)c : (i64)c);
+}
+
+// recon6's *lost for either sign of a scalar's differences x +- g, told before the
+// reconstructions (a flag after them keeps the FP64 differences in registers all
+// the while: 96 instead of 64, 13695 x 5 Burgers cells 60.4 -> 64.6 us a step).
+WENO_FX bool lost_pair(const i64 (&x)[5], const i64 (&g)[5]) {
+  bool flat = false;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) flat = flat || (x[j] | g[j] | x[j + 1] | g[j + 1]) == 0;
+  if (!flat) return false;
+  const i64 a = (x[0] + x[4]) - 4 * (x[1] + x[3]) + 6 * x[2];
+  const i64 b = (g[0] + g[4]) - 4 * (g[1] + g[3]) + 6 * g[2];
+  i64 p = 0, n = 0;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    p |= x[j] + g[j];
+    n |= x[j] - g[j];
+  }
+  return (p != 0 && abs64(a + b) < (1ull << 29)) || (n != 0 && abs64(a - b) < (1ull << 29));
 }
 
 // The largest biased exponent of the ten differences.
@@ -327,7 +353,6 @@ WENO_FX Limb coefficient(double x, int E, int um) {
   return limb((i64)b < 0 ? -(i64)v : (i64)v);
 }
 WENO_FX int exponent(double x) { return (int)((hi32(dbits(x)) >> 20) & 0x7FF); }
-WENO_FX int imax(int a, int b) { return a > b ? a : b; }
 // A GLF speed A < 2^a as A 2^(63 - a).
 WENO_FX Limb speed(double A, int a) {
   const u64 b = dbits(A);
@@ -597,7 +622,9 @@ WENO_FX bool smooth_term(const i64 (&d)[5], int &corr) {
   const float b2 = ffma(fmul(13.0f, a2), a2, fmul(fmul(3.0f, t2), t2));
   const float bd = ffma(fmul(13.0f, a3), a3, fmul(fmul(3.0f, t3), t3));
   const float b3 = fmul(0.25f, fadd(fadd(b0, b1), fadd(b2, bd)));
-  const float T = fmul(fmul(12.0f, r5), r5), T9 = fmul(9.0f, T), tiny = 1e-30f;
+  // (2^-126 / 2^-120: an indicator of 0 beside r5 = 0 gives G = 9 / 64, so that
+  // recon6 decides there unless the candidates agree to 2^6 units)
+  const float T = ffma(fmul(12.0f, r5), r5, 0x1p-126f), T9 = fmul(9.0f, T), tiny = 0x1p-120f;
   const float g0 = fmul(T, rcpf(fadd(b0, tiny))), g1 = fmul(T9, rcpf(fadd(b1, tiny)));
   const float g2 = fmul(T9, rcpf(fadd(b2, tiny))), g3 = fmul(T, rcpf(fadd(b3, tiny)));
   // r_k - r_1, their mean m, and r_k - rm

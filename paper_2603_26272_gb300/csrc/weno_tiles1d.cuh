@@ -284,7 +284,7 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     const bool act = (f <= T) && (i0 + f - 1 < nx);
     double dw[5] = {}, dg[5] = {}, xw[5] = {};
     double A = 0.0, base = 0.0;
-    bool fixed = false, flat = false;
+    bool fixed = false, flat = false, lost = false;
     fx::i64 c = 0;
     const ReconParams &rp = s_rp[0];
     double scale = 0.0;
@@ -301,15 +301,23 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
       if constexpr (P1) {
         const int es = fx::top_exponent(xw, dg);
         fixed = es >= rp.es_lo && es <= rp.es_hi && !fx::uneven(xw, dg, es, centre);
+        fx::i64 x[5], g[5];
+        if (fixed) {
+#pragma unroll
+          for (int j = 0; j < 5; ++j) {
+            x[j] = fx::to_fixed(xw[j], es);
+            g[j] = fx::to_fixed(dg[j], es);
+          }
+          fixed = !fx::lost_pair(x, g);
+        }
         if (fixed) {
           fx::i64 d[5];
 #pragma unroll
           for (int j = 0; j < 5; ++j) {
-            const fx::i64 x = fx::to_fixed(xw[j], es), g = fx::to_fixed(dg[j], es);
             if (sgn)
-              d[4 - j] = x - g;
+              d[4 - j] = x[j] - g[j];
             else
-              d[j] = x + g;
+              d[j] = x[j] + g[j];
           }
           c = recon_fixed<AI>(d, es - 1079, rp);
           scale = fx::scale_back(es);
@@ -324,7 +332,9 @@ __device__ __forceinline__ void line1d_tile(const StageArgs &a, long long b, lon
     }
     c += __shfl_xor_sync(0xffffffffu, c, 1);
     double h = flat ? base : __fma_rn((double)c, scale, base);
-    const bool wide = act && !fixed && !flat;
+    // (a flux that the integer path gives up takes its face along)
+    const unsigned gone = __ballot_sync(0xffffffffu, lost) >> (tid & 30) & 3u;
+    const bool wide = act && !flat && (!fixed || gone != 0);
     if (__any_sync(0xffffffffu, wide)) {
       ZA6Part part = {0.0, 1.0};
       if (wide) part = recon_wide<AI, P1>(dw, dg, A, sgn, rp);

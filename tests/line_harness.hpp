@@ -217,9 +217,14 @@ void fields_fixed(const Line<NC> &s, const Cell<double> *x, const Face<double> &
     if (sh == 64) continue;
     shift_field(X, sh);
     shift_field(G, sh);
-    const i64 S = rough_sum(X, G, [](const i64(&e)[5]) {
-      return recon6<false>(e[0], e[1], e[2], e[3], e[4], Flt()); });
+    bool lost = false;
+    const i64 S = rough_sum(X, G, [&](const i64(&e)[5]) {
+      return recon6<false>(e[0], e[1], e[2], e[3], e[4], Flt(), &lost); });
     h[m] = from_fixed(S, k0 + 6 - sh) / 6;
+    if (lost) {
+      fields<double, NC>(s, x, f, A, i0, wide);
+      h[m] = wide[m];
+    }
   }
 }
 template <class T, int NC>

@@ -302,15 +302,18 @@ __device__ __forceinline__ float speed_floor(const unsigned long long *slot, int
 // True where the state is physical and none of its speeds can reach its floor,
 // with a margin of 2^-9 of the speeds for the FP32 arithmetic (p above 2^-12 E,
 // so the sound speed is good to 2^-11); false (FP64 decides) for anything else,
-// NaN and magnitudes near FP32's limits included.
+// NaN and magnitudes near FP32's limits included: c^2 has to be a normal number
+// (a cold, dense cell's is flushed to 0, and its c would be missing).
 __device__ __forceinline__ bool speeds_below(double rho, double mx, double my, double E, float gg,
                                              const float *floors) {
   const float r = f32_rn(rho), m = f32_rn(mx), n = f32_rn(my), e = f32_rn(E);
   const float ir = fx::rcpf(r), u = m * ir, v = n * ir;
   const float pe = e - 0.5f * (m * u + n * v);
   if (!(r > 1e-18f && r < 1e18f && e > 1e-18f && e < 1e18f && pe > e * 0x1p-12f)) return false;
+  const float cc = gg * pe * ir;
+  if (!(cc >= 0x1p-126f)) return false;
   float c;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(gg * pe * ir));
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(cc));
   const float mg = 0x1p-9f * (fmaxf(fabsf(u), fabsf(v)) + c);
   return fabsf(u - c) + mg < floors[0] && fabsf(u) + mg < floors[1] &&
          fabsf(u + c) + mg < floors[2] && fabsf(v - c) + mg < floors[3] &&

@@ -122,6 +122,12 @@ struct StageArgs {
   // wait, WENO_TEST_TMA_NO_COPY=1 in the environment) arms the barrier but
   // issues no copy, so every TMA wait runs out and reports WENO_ERR_TIMEOUT
   int use_tma, tma_no_copy;
+  // 2D: filter the cells by FP32 estimates of their speeds (speeds_below).  Not
+  // where every block has an SM alone: they reach their last phase together, with
+  // no maxima to compare with yet (steps of 64^2 and 96^2, FP32 reconstruction:
+  // 89.5 -> 86.9 and 96.1 -> 93.2 us; with more blocks on an SM the later ones do
+  // find some: 320^2 without the filter 302 -> 312 us).  Set by the launcher.
+  int speed_filter;
 };
 
 // Wavespeed reduction of U into alpha_out (which must be zero), optional dt.

@@ -170,6 +170,7 @@ __device__ __forceinline__ StageArgs slot_stage_args(const SlotDev &S, int stage
   a.halo_lo = a.halo_hi = nullptr;
   a.send_lo = a.send_hi = nullptr;
   a.use_tma = a.tma_no_copy = 0;
+  a.speed_filter = 1;
   a.sp_at = &S.sp;
   a.t = S.clock;
   a.tnext = S.clock + 1;

@@ -335,8 +335,9 @@ __device__ __forceinline__ void tile2d_update(const StageArgs &a, long long b, l
   unsigned long long mx6[6] = {0ull, 0ull, 0ull, 0ull, 0ull, 0ull};
   const bool want_alpha = (a.mode == 0) && (a.alpha_out != nullptr);
   const float gg = (float)(a.gamma * gm1);
+  const bool filter = want_alpha && a.speed_filter;
   __shared__ float floors[6];
-  if (want_alpha) {
+  if (filter) {
     if (tid < 6) floors[tid] = speed_floor(a.alpha_out + b * 8, tid);
     __syncthreads();
   }
@@ -367,7 +368,7 @@ __device__ __forceinline__ void tile2d_update(const StageArgs &a, long long b, l
     if (a.send_hi && gj >= a.ny - R)
 #pragma unroll
       for (int q = 0; q < 4; ++q) a.send_hi[((b * 4 + q) * R + (gj - (a.ny - R))) * a.nx + gi] = uo[q];
-    if (want_alpha && !speeds_below(uo[0], uo[1], uo[2], uo[3], gg, floors)) {
+    if (want_alpha && !(filter && speeds_below(uo[0], uo[1], uo[2], uo[3], gg, floors))) {
       const double ir = rcp_pos(uo[0]);
       const double u = uo[1] * ir, v = uo[2] * ir;
       const double p = gm1 * (uo[3] - 0.5 * fma(uo[1], u, uo[2] * v));
@@ -864,7 +865,7 @@ __device__ __forceinline__ void euler2d_tile6(const StageArgs &a, long long b, l
   __shared__ SchemeParams s_scheme;
   load_scheme(a, s_scheme);
   __shared__ Speeds s_sp;
-  make_speeds(a, b, 4, s_sp);
+  if constexpr (P1 && PREC == 0) make_speeds(a, b, 4, s_sp);
 
   const bool use_tma = tm != nullptr && i0 - XO >= 0 && i0 - XO + BW <= a.nx && j0 - R >= 0 &&
                        j0 + TY + R <= a.ny;
@@ -1021,6 +1022,7 @@ cudaError_t launch_2d(const StageArgs &a_in, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long tiles = ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY);
   dim3 grid((unsigned)tiles, 1, (unsigned)a.nbatch);
+  a.speed_filter = tiles * a.nbatch > (long long)sm_count();
   return launch_chained(fits(grid, 2), kern, grid, NT, smem, s, a, tm);
 }
 

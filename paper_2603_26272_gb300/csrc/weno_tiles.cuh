@@ -22,6 +22,7 @@
 //      characteristic speeds, reduced with warp shuffles and one atomicMax
 //      per value and block.
 #pragma once
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <cstdlib>
@@ -1031,12 +1032,20 @@ inline long long tiles_2d(const StageArgs &a) {
   return ((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY) * a.nbatch;
 }
 
-// What a stage of `tiles` tiles costs that give every thread `faces` faces, in
-// tenths of a face of a full wave: a face takes 127 us (r = 5) where per_sm
-// blocks share an SM and 77 where one has it alone.
-inline long long wave_cost(long long tiles, int faces, int per_sm) {
-  const long long wave = (long long)sm_count() * per_sm, rest = tiles % wave;
-  return faces * (10 * (tiles / wave) + (rest == 0 ? 0 : rest <= sm_count() ? 6 : 10));
+// What a stage of the tiles (TX, TY) costs, orders 4, 8 and 10, with blocks
+// that come in rounds of one an SM: `two` for a pair of rounds, `one` for a single
+// one.  Measured in 1/40 of a pair of 16x15 (r = 5, right-hand sides of 48 grids
+// from 48 to 1024 cells a side): 300 us the first round, 555 a pair, the same on the
+// 20x15 tiles 375 and 690, on 16x16 370 and 620, 97 each round of 8x8 tiles, and r = 4
+// in the same proportions; r = 2, three blocks an SM, 80 each round of 16x15, 84 of
+// 16x16, 100 of 20x15, 26 of 8x8.
+template <int TX, int TY, int R>
+inline long long tiles_cost(const StageArgs &a) {
+  constexpr int two = R == 2 ? (TX == 8 ? 26 : TX == 20 ? 100 : TY == 16 ? 84 : 80)
+                             : (TX == 8 ? 14 : TX == 20 ? 50 : TY == 16 ? 45 : 40);
+  constexpr int one = R == 2 || TX == 8 ? two / 2 : (TX == 20 || TY == 16 ? 27 : 22);
+  const long long rounds = (tiles_2d<TX, TY>(a) + sm_count() - 1) / sm_count();
+  return rounds / 2 * two + rounds % 2 * one;
 }
 
 template <int AI, bool P1, int PREC, int R>
@@ -1059,28 +1068,25 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     // Weights other than the default ones (without Ai, with a sensitivity term
     // that counts, p != 1) are built in three of the shapes (2, 8, 9; see
     // tile_shape_built), which keeps the library's build short.
-    // The other orders use 16x15 / 128, 3 blocks per SM at r = 2 and 2 at
-    // r = 4, 5 (their wider stencils need more registers): 511 faces, four a
-    // thread, where 16x16 has 544 and every block's warp 0 a fifth round of them
-    // on the same sub-partition (300^2 steps of orders 4 / 8 / 10: 830 / 2112 /
-    // 3027 -> 755 / 1826 / 2605 us; 1024 x 512, orders 8 / 10: 9.10 / 13.07 ->
-    // 8.72 / 12.50 ms).  A grid of no more such tiles than SMs, where a stage
-    // lasts as long as one thread's faces, takes 8x8 / 160 (144 faces, one a
-    // thread): 64^2, orders 8 / 10: 812 / 1158 -> 230 / 314 us; 150^2 (100 of the
-    // large tiles): 811 / 1159 -> 657 / 909 us.  Above that line the halo costs
-    // more than the length gives.
-    // Between them, the shape whose last wave is fuller: 20x15 / 128 (635 faces,
-    // five a thread) where wave_cost says so (orders 8 / 10, 16x15 -> 20x15:
-    // 220x190 1193 / 1694 -> 834 / 1182 us, 300^2 1826 / 2605 -> 1493 / 2120,
-    // 512^2 4659 / 6657 -> 4378 / 6253).
+    // The other orders run 3 blocks per SM at r = 2 and 2 at r = 4, 5 (their
+    // wider stencils need more registers) in the shape whose rounds cost least
+    // (tiles_cost): 16x15 / 128 (511 faces, four a thread), 16x16 / 128 (544: a fifth
+    // round for warp 0 alone, but fewer tiles), 20x15 / 128 (635, five a thread), 8x8 /
+    // 160 (144, one a thread, for grids where a stage lasts as long as one thread's
+    // faces).  Right-hand sides of order 10 in the four, us: 512^2 (1120, 1024, 910,
+    // 4096 tiles) 2226 / 2238 / 2089 / 2746; 192x161 319 / 389 / 395 / 400; 100x649 866 /
+    // 638 / 707 / 784; 306x140 570 / 635 / 705 / 498; the rule takes the least in all
+    // 48 grids at orders 8 and 10, and loses 0.4 % to it at order 4.
     if constexpr (R != 3) {  // r = 2 fits the 168-register cap of 3 blocks per SM
       constexpr int kPerSM = R == 2 ? 3 : 2;
+      const long long c15 = tiles_cost<16, 15, R>(a), c16 = tiles_cost<16, 16, R>(a);
       if constexpr (P1) {
-        if (tiles_2d<16, 15>(a) <= sm_count())
-          return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
-        if (wave_cost(tiles_2d<20, 15>(a), 5, kPerSM) < wave_cost(tiles_2d<16, 15>(a), 4, kPerSM))
-          return launch_2d<20, 15, 128, kPerSM, AI, P1, PREC, R>(a, s);
+        const long long c20 = tiles_cost<20, 15, R>(a), c8 = tiles_cost<8, 8, R>(a);
+        const long long large = std::min(c15, std::min(c16, c20));
+        if (c8 < large) return launch_2d<8, 8, 160, 1, AI, P1, PREC, R>(a, s);
+        if (c20 < std::min(c15, c16)) return launch_2d<20, 15, 128, kPerSM, AI, P1, PREC, R>(a, s);
       }
+      if (c16 < c15) return launch_2d<16, 16, 128, kPerSM, AI, P1, PREC, R>(a, s);
       return launch_2d<16, 15, 128, kPerSM, AI, P1, PREC, R>(a, s);
     } else if constexpr (!all_tile_shapes(AI, P1, PREC)) {
       switch (tile_shape_built(false, a.tile_variant)) {

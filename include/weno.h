@@ -111,7 +111,7 @@ weno_status weno_wavespeeds(const weno_desc *d, const double *U, double *alpha, 
 /* Tile autotuning (2D, order 6).  weno_rhs, weno_step and weno_solve choose
  * among eleven tile shapes of the 2D stage kernel (all give bitwise the same
  * result; weights other than the default ones -- ai = 0, a larger epsilon or
- * mu0, p != 1 -- have three of them, for which the other numbers stand).  The
+ * mu0, p != 1 -- have four of them, for which the other numbers stand).  The
  * first such call on a new problem shape (nx, ny, nbatch,
  * precision, ai, p == 1, and in FP64 with ai = 1 and p = 1 whether eps <= 2^-126
  * and mu0 <= 2^-100) in a process times them on the caller's data: two

@@ -292,7 +292,7 @@ weno_status read_status(const Ctx &c) {
 // stage each, written into the scratch state U1) and caches the fastest; all
 // variants compute bitwise the same result.  WENO_TILE2D=0..10 in the
 // environment forces a variant and skips the timing.  Weights other than the
-// default ones have three shapes built; the other numbers stand for one of them
+// default ones have four shapes built; the other numbers stand for one of them
 // (tile_shape_built).
 // ---------------------------------------------------------------------------
 std::mutex g_tune_mu;

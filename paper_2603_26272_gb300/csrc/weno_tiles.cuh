@@ -1066,7 +1066,7 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     // FP64 pipes idle at the end of a sweep): 9 = 16x15 / 128 / 3 (255 and
     // 256 faces), 10 = 14x17 / 128 / 3 (255 and 252).
     // Weights other than the default ones (without Ai, with a sensitivity term
-    // that counts, p != 1) are built in three of the shapes (2, 8, 9; see
+    // that counts, p != 1) are built in four of the shapes (2, 7, 8, 9; see
     // tile_shape_built), which keeps the library's build short.
     // The other orders run 3 blocks per SM at r = 2 and 2 at r = 4, 5 (their
     // wider stencils need more registers) in the shape whose rounds cost least
@@ -1091,6 +1091,7 @@ cudaError_t launch_stage_t(const StageArgs &a, cudaStream_t s) {
     } else if constexpr (!all_tile_shapes(AI, P1, PREC)) {
       switch (tile_shape_built(false, a.tile_variant)) {
         case 2: return launch_2d<16, 8, 64, 4, AI, P1, PREC>(a, s);
+        case 7: return launch_2d<16, 8, 256, 1, AI, P1, PREC>(a, s);
         case 8: return launch_2d<8, 8, 128, 2, AI, P1, PREC>(a, s);
         default: return launch_2d<16, 15, 128, 3, AI, P1, PREC>(a, s);
       }

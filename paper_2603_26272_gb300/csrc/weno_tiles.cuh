@@ -219,8 +219,21 @@ __device__ __forceinline__ void tma_issue_box(const CUtensorMap *tm, unsigned ba
 }
 
 // SM clock cycles a TMA wait may take before it gives up (about 1 ms at
-// 2 GHz; the copy of one box takes microseconds).
-constexpr long long kTmaWaitCycles = 2000000;
+// 2 GHz; the copy of one box takes microseconds).  The clock runs on while another
+// process has the GPU, so that a poll that was interrupted would use them all up (four
+// processes at once saw WENO_ERR_TIMEOUT): no more than kTmaPollCycles of it count
+// between two polls.
+constexpr long long kTmaWaitCycles = 2000000, kTmaPollCycles = 20000;
+__device__ __forceinline__ bool tma_wait(unsigned bar) {
+  long long left = kTmaWaitCycles, t = clock64();
+  bool done;
+  while (!(done = mbar_try_wait(bar, 0)) && left > 0) {
+    const long long now = clock64(), dt = now - t;
+    left -= dt > 0 && dt < kTmaPollCycles ? dt : kTmaPollCycles;
+    t = now;
+  }
+  return done;
+}
 
 // The TMA copy of tile (i0, j0)'s box of problem b into `box` (every thread
 // of the block calls this).  Returns false -- after recording
@@ -247,15 +260,10 @@ __device__ bool tma_stage_box(const StageArgs &a, const CUtensorMap *tm, double 
       tma_issue_box(tm, bar, box, (int)(i0 - TmaBox<R>::XO), (int)(j0 - R), (int)(b * 4),
                     (unsigned)tma_box_bytes<TX, TY, R>());
   }
-  long long t_start = clock64();
-  bool done = false;
-  while (!(done = mbar_try_wait(bar, 0)) && clock64() - t_start < kTmaWaitCycles) {
-  }
+  const bool done = tma_wait(bar);
   if (!__syncthreads_and(done)) {
     if (tid == 0) record_status(a.status, 5, a.stage, b, j0, i0);
-    t_start = clock64();
-    while (!mbar_try_wait(bar, 0) && clock64() - t_start < kTmaWaitCycles) {
-    }
+    tma_wait(bar);
     return false;
   }
   return true;

@@ -51,7 +51,8 @@ FLOPS_PER_CELL_STAGE = FLOPS_PER_CELL_UPDATE / 3.0
 # (32 B), stages 2 and 3 also read U^n, and each writes its output:
 # 32 x (2 + 3 + 3) = 256 B.
 BYTES_PER_CELL_UPDATE = 256.0
-KERNEL_SOURCES = ["paper_2603_26272_gb300/csrc/weno_tiles.cuh",
+KERNEL_SOURCES = ["paper_2603_26272_gb300/csrc/weno_fixed.cuh",
+                  "paper_2603_26272_gb300/csrc/weno_tiles.cuh",
                   "paper_2603_26272_gb300/csrc/weno_kernels.cu",
                   "paper_2603_26272_gb300/csrc/weno_device.cuh"]
 

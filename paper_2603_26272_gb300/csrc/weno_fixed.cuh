@@ -17,10 +17,11 @@
 // Measured at 2048^2, FP64, one step: 33.5 ms with the reconstruction and the
 // projections on the FP64 pipe, 16.0 ms with the reconstruction here, 9.16 ms
 // with the projections (project) and the smooth stencils (smooth_term) too,
-// 7.85 ms with the scheme's constants from the host and the speed maxima
-// filtered in FP32.  What is left is bound by both: FP64 pipe 57 %, integer
-// (alu) 36 %, 44 % of the issue slots (1024^2, 11.3k instructions and 214 FP64
-// operations per cell and stage).
+// 7.87 ms with the scheme's constants from the host and the speed maxima
+// filtered in FP32, 7.95 ms with a scale for each group of fields and with what
+// a common unit does not serve left to FP64.  What is left is bound by both: FP64
+// pipe 56 %, integer (alu) 38 %, 48 % of the issue slots (1024^2, 11.8k instructions
+// and 211 FP64 operations per cell and stage).
 //
 // Number formats (tests/test_kernel_fixed.py compiles this header for the host
 // and measures the error against quadruple precision):
